@@ -79,6 +79,7 @@ LcModel<T> lc_model_of(const lc_params& p) {
     m.fm.force_pre = (T)(1.0 - 0.5 / p.tau_f);
     m.fm.omega_m = m.fm.omega_f;
     m.fm.force_pre_m = m.fm.force_pre;
+    m.fm.pc = ld::pair_coef_of<T>(1.0 / p.tau_f, 1.0 - 0.5 / p.tau_f, 1.0 / p.tau_f, 1.0 - 0.5 / p.tau_f, 0.0, 0.0);
     return m;
 }
 
@@ -267,13 +268,8 @@ __device__ __forceinline__ void lc_stress(const A (&q)[6], const A (&dQ)[3][6], 
 // uv.
 template <class T>
 __device__ __forceinline__ void lc_moments_u(const T (&fv)[Q], const T (&Fa)[3], T& rho, T (&uv)[3]) {
-    T jx = T(0), jy = T(0), jz = T(0);
-    rho = T(0);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        rho += fv[i];
-        ld::add_c(i, fv[i], jx, jy, jz);
-    }
+    T jx, jy, jz;
+    ld::moments_f(fv, rho, jx, jy, jz);
     ld::guo_velocity(rho, jx, jy, jz, Fa[0], Fa[1], Fa[2], uv[0], uv[1], uv[2]);
 }
 template <class T>

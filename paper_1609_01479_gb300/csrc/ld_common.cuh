@@ -164,6 +164,21 @@ struct Geom {
     long long n, npad;
 };
 
+// Products of the relaxation constants and the diagonal weight w = 1/36 that
+// the FP64 collisions use, formed once on the host: on the FP64 pipe, which
+// bounds the FP64 step, each would cost every thread an instruction.
+// omega, pre: of the even parts (all of f in BGK); omega_m, pre_m: of the
+// odd parts (the same in BGK).
+template <class R>
+struct PairCoef {
+    R keep_f, keep_g;  // 1 - omega_f, 1 - omega_g
+    R half_p, half_m;  // (1 - omega)/2, (1 - omega_m)/2
+    R f_odd;           // 3 w omega_m
+    R src3, src9;      // -3 pre, 9 w pre
+    R src_odd;         // 3 w pre_m
+    R g_mu, g_phi;     // 9/2 w omega_g Gamma, -3/2 w omega_g
+};
+
 // Model constants in the arithmetic type.
 template <class R>
 struct Model {
@@ -174,7 +189,26 @@ struct Model {
     int trt;             // 1: two-relaxation-time collision of f (LD_COLLISION_TRT)
     R omega_m;           // TRT: 1/tau- of the odd parts
     R force_pre_m;       // TRT: 1 - 1/(2 tau-)
+    PairCoef<R> pc;
 };
+
+// PairCoef from the relaxation rates (omega_g, Gamma: 0 where there is no g).
+template <class R>
+inline PairCoef<R> pair_coef_of(double omega_f, double pre, double omega_m, double pre_m, double omega_g,
+                                double Gamma) {
+    PairCoef<R> c;
+    c.keep_f = (R)(1.0 - omega_f);
+    c.keep_g = (R)(1.0 - omega_g);
+    c.half_p = (R)(0.5 * (1.0 - omega_f));
+    c.half_m = (R)(0.5 * (1.0 - omega_m));
+    c.f_odd = (R)(omega_m / 12.0);
+    c.src3 = (R)(-3.0 * pre);
+    c.src9 = (R)(0.25 * pre);
+    c.src_odd = (R)(pre_m / 12.0);
+    c.g_mu = (R)(0.125 * omega_g * Gamma);
+    c.g_phi = (R)(omega_g / -24.0);
+    return c;
+}
 
 // Model constants from the C-ABI parameters.
 template <class R>
@@ -192,6 +226,7 @@ inline Model<R> model_of(const ld_params& p) {
     const double tau_m = m.trt ? 0.5 + p.magic / (p.tau_f - 0.5) : p.tau_f;
     m.omega_m = (R)(1.0 / tau_m);
     m.force_pre_m = (R)(1.0 - 0.5 / tau_m);
+    m.pc = pair_coef_of<R>(1.0 / p.tau_f, 1.0 - 0.5 / p.tau_f, 1.0 / tau_m, 1.0 - 0.5 / tau_m, 1.0 / p.tau_g, p.Gamma);
     return m;
 }
 
@@ -220,10 +255,20 @@ __device__ __forceinline__ R chem_potential_lap(R phi, R lap, const Model<R>& m)
     return sub_rn(add_rn(mul_rn(m.A, phi), cubic), mul_rn(m.kappa, lap));
 }
 
+// FP64, where each operation costs the pipe that bounds the step: phi (A +
+// B phi^2) - kappa lap in four instructions instead of seven.
+__device__ __forceinline__ double chem_potential_lap(double phi, double lap, const Model<double>& m) {
+    return __fma_rn(phi, __fma_rn(m.B, __dmul_rn(phi, phi), m.A), -__dmul_rn(m.kappa, lap));
+}
+
+// 7-point lap from the sum of the six axis neighbours: nb_sum - 6 h.
+__device__ __forceinline__ float lap7(float h, float nb_sum) { return sub_rn(nb_sum, mul_rn(6.0f, h)); }
+__device__ __forceinline__ double lap7(double h, double nb_sum) { return __fma_rn(-6.0, h, nb_sum); }
+
 // The same with the 7-point lap = (sum of the six axis neighbours' phi) - 6 phi.
 template <class R>
 __device__ __forceinline__ R chem_potential(R phi, R nb_sum, const Model<R>& m) {
-    return chem_potential_lap(phi, sub_rn(nb_sum, mul_rn(R(6), phi)), m);
+    return chem_potential_lap(phi, lap7(phi, nb_sum), m);
 }
 
 // 19-point isotropic forms on the D3Q19 neighbourhood. nb(i) is h(x + c_i).
@@ -293,14 +338,52 @@ __device__ __forceinline__ void add_c(int i, R v, R& jx, R& jy, R& jz) {
     if (cz(i) < 0) jz -= v;
 }
 
+// rho = sum f_i and j = sum f_i c_i of one site. FP32 accumulates direction
+// by direction. FP64 forms j from the opposite pairs' differences, 39
+// operations instead of 48, with rho in the same order.
+__device__ __forceinline__ void moments_f(const float (&f)[Q], float& rho, float& jx, float& jy, float& jz) {
+    rho = jx = jy = jz = 0.0f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        rho += f[i];
+        add_c(i, f[i], jx, jy, jz);
+    }
+}
+__device__ __forceinline__ void moments_f(const double (&f)[Q], double& rho, double& jx, double& jy, double& jz) {
+    rho = f[0];
+#pragma unroll
+    for (int i = 1; i < Q; ++i) rho += f[i];
+    jx = f[1] - f[2];
+    jy = f[3] - f[4];
+    jz = f[5] - f[6];
+#pragma unroll
+    for (int i = 7; i < Q; i += 2) add_c(i, f[i] - f[i + 1], jx, jy, jz);
+}
+
+// F = -phi gm from the unscaled central differences d = 2 gm (7-point form):
+// -phi (d/2) and (-phi/2) d are the same values, halving being exact.
+template <class R>
+__device__ __forceinline__ void force_of_diffs(R phi, R dx, R dy, R dz, R& Fx, R& Fy, R& Fz) {
+    const R h = R(-0.5) * phi;
+    Fx = h * dx;
+    Fy = h * dy;
+    Fz = h * dz;
+}
+
 // Guo velocity from the moments and the force: u = (j + F/2) / rho. FP64
-// divides (the rounding the FP64 path is held to); FP32 multiplies by the
-// correctly rounded reciprocal.
+// takes one reciprocal and corrects each quotient by its residual (two fused
+// operations), which leaves the error of a division; three divisions took 28
+// FP64 instructions. FP32 multiplies by the correctly rounded reciprocal.
+__device__ __forceinline__ double div_by(double n, double d, double inv) {
+    const double q = __dmul_rn(n, inv);
+    return __fma_rn(__fma_rn(-q, d, n), inv, q);
+}
 __device__ __forceinline__ void guo_velocity(double rho, double jx, double jy, double jz, double Fx, double Fy,
                                              double Fz, double& ux, double& uy, double& uz) {
-    ux = (jx + 0.5 * Fx) / rho;
-    uy = (jy + 0.5 * Fy) / rho;
-    uz = (jz + 0.5 * Fz) / rho;
+    const double inv = __drcp_rn(rho);
+    ux = div_by(__fma_rn(0.5, Fx, jx), rho, inv);
+    uy = div_by(__fma_rn(0.5, Fy, jy), rho, inv);
+    uz = div_by(__fma_rn(0.5, Fz, jz), rho, inv);
 }
 __device__ __forceinline__ void guo_velocity(float rho, float jx, float jy, float jz, float Fx, float Fy, float Fz,
                                              float& ux, float& uy, float& uz) {
@@ -310,67 +393,76 @@ __device__ __forceinline__ void guo_velocity(float rho, float jx, float jy, floa
     uz = (jz + 0.5f * Fz) * inv;
 }
 
-// BGK + Guo collision of f in place.
-//
-// The generic template evaluates the equilibrium and the source term
-// direction by direction, in the operation order of the formulas above.
-// FP64 and FP32 (also the arithmetic of the 16-bit forms) use specialisations
-// on opposite pairs (i, i+1), c_{i+1} = -c_i: c.u and c.F change sign within
-// a pair, so
+// BGK + Guo collision of f in place, on opposite pairs (i, i+1), c_{i+1} =
+// -c_i: c.u and c.F change sign within a pair, so
 //   feq_(i,i+1) = w rho (1 - 3/2 u.u + 9/2 (c.u)^2) +- 3 w rho c.u
 //   src_(i,i+1) = pre w (9 (c.u)(c.F) - 3 u.F)        +- 3 pre w c.F
-// and each pair shares its symmetric part. In FP32 the rest equilibrium is
-// rho minus the 18 moving ones (the same value in exact arithmetic): the
-// nearest floats to 1/3, 1/18, 1/36 sum to 1 + 1.5e-8, and the formula for
-// every direction would add that much mass to each site at every step.
+// and each pair shares its symmetric part. In FP32 (also the arithmetic of
+// the 16-bit forms) the rest equilibrium is rho minus the 18 moving ones (the
+// same value in exact arithmetic): the nearest floats to 1/3, 1/18, 1/36 sum
+// to 1 + 1.5e-8, and the formula for every direction would add that much
+// mass to each site at every step.
 template <class R>
 __device__ __forceinline__ void collide_f(R (&f)[Q], R rho, R ux, R uy, R uz, R Fx, R Fy, R Fz,
-                                          const Model<R>& m) {
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        const R cu = cdot(i, ux, uy, uz);
-        const R cF = cdot(i, Fx, Fy, Fz);
-        const R feq = wgt<R>(i) * rho * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-        const R src = m.force_pre * wgt<R>(i) * (R(3) * (cF - uF) + R(9) * cu * cF);
-        f[i] = f[i] - m.omega_f * (f[i] - feq) + src;
-    }
-    // c_0 = 0: feq_0 = w_0 rho (1 - 3/2 u.u), src_0 = pre w_0 (-3 u.F)
-    const R feq0 = wgt<R>(0) * rho * (R(1) - R(1.5) * uu);
-    const R src0 = m.force_pre * wgt<R>(0) * (R(3) * (-uF));
-    f[0] = f[0] - m.omega_f * (f[0] - feq0) + src0;
-}
+                                          const Model<R>& m);
 
-// FP64 on opposite pairs too (with the g collision's pair form, about 35 %
-// fewer FP64 operations per site than direction by direction, where the FP64
-// pipe is the bound); the rest
-// equilibrium from its formula, the FP64 weights summing to 1 within an ulp.
+// The FP64 collision of f, BGK or TRT (see collide_f_trt). The FP64 pipe
+// (two instructions per clock and SM) bounds the FP64 step, so the pairs are
+// written for the fewest instructions. The equilibrium and the source term
+// enter a pair only through
+//   even  w a + (c.u)(c.e),  e = 9/2 w omega rho u + 9 w pre F,
+//         a = omega rho (1 - 3/2 u.u) - 3 pre u.F,
+//   odd   c.o,               o = 3 w omega_m rho u + 3 w pre_m F,
+// so the vectors e and o are formed once per site and a diagonal pair costs
+// eight instructions (BGK), an axis pair, whose weight is twice the diagonal
+// one, five on the doubled vectors (doubling is exact). The rest population
+// takes a/3. No constant carries omega times a weight where mass depends on
+// it (9/2 w = 1/8 exactly; w and 1/3 multiply a as they stand): with w omega
+// rounded once on the host the sum of the weights would be off by up to 1e-16,
+// and so would the mass after every step. With the g collision, the moments
+// and the velocity in the same manner a site takes about 265 FP64
+// instructions in a whole step, down from 495; the step at 128^3 takes 0.99 ms
+// (1.97 before). Measured against 128-bit arithmetic on random sites, tau =
+// 0.8: relative error of f 2.19e-16 and of g 2.76e-16 (separate equilibrium
+// and source terms: 2.25e-16 and 3.05e-16), mean change of mass -6e-17 (the
+// same).
+template <bool TRT>
+__device__ __forceinline__ void collide_f_pairs(double (&f)[Q], double rho, double ux, double uy, double uz, double Fx,
+                                                double Fy, double Fz, double omega, const PairCoef<double>& k) {
+    const double uu = __fma_rn(ux, ux, __fma_rn(uy, uy, __dmul_rn(uz, uz)));
+    const double uF = __fma_rn(ux, Fx, __fma_rn(uy, Fy, __dmul_rn(uz, Fz)));
+    const double p = omega * rho;
+    const double a = __fma_rn(p, __fma_rn(-1.5, uu, 1.0), k.src3 * uF);
+    const double wa = wgt<double>(7) * a;
+    const double re = 0.125 * p, ro = k.f_odd * rho;
+    const double ex = __fma_rn(re, ux, k.src9 * Fx), ey = __fma_rn(re, uy, k.src9 * Fy),
+                 ez = __fma_rn(re, uz, k.src9 * Fz);
+    const double ox = __fma_rn(ro, ux, k.src_odd * Fx), oy = __fma_rn(ro, uy, k.src_odd * Fy),
+                 oz = __fma_rn(ro, uz, k.src_odd * Fz);
+    auto put = [&](int i, double even, double odd) {
+        if (TRT) {
+            const double np = __fma_rn(k.half_p, f[i] + f[i + 1], even);
+            const double nm = __fma_rn(k.half_m, f[i] - f[i + 1], odd);
+            f[i] = np + nm;
+            f[i + 1] = np - nm;
+        } else {
+            f[i] = __fma_rn(k.keep_f, f[i], even + odd);
+            f[i + 1] = __fma_rn(k.keep_f, f[i + 1], even - odd);
+        }
+    };
+    f[0] = __fma_rn(wgt<double>(0), a, k.keep_f * f[0]);
+    const double A2 = wa + wa;
+    put(1, __fma_rn(ux, ex + ex, A2), ox + ox);
+    put(3, __fma_rn(uy, ey + ey, A2), oy + oy);
+    put(5, __fma_rn(uz, ez + ez, A2), oz + oz);
+#pragma unroll
+    for (int i = 7; i < Q; i += 2)
+        put(i, __fma_rn(cdot(i, ux, uy, uz), cdot(i, ex, ey, ez), wa), cdot(i, ox, oy, oz));
+}
 template <>
 __device__ __forceinline__ void collide_f<double>(double (&f)[Q], double rho, double ux, double uy, double uz,
                                                   double Fx, double Fy, double Fz, const Model<double>& m) {
-    const double uu = ux * ux + uy * uy + uz * uz;
-    const double uF = ux * Fx + uy * Fy + uz * Fz;
-    const double base = 1.0 - 1.5 * uu;
-    const double keep = 1.0 - m.omega_f;
-#pragma unroll
-    for (int i = 1; i < Q; i += 2) {
-        const double w = wgt<double>(i);
-        const double wr = w * rho, pw = m.force_pre * w;
-        const double cu = cdot(i, ux, uy, uz);
-        const double cF = cdot(i, Fx, Fy, Fz);
-        const double feq_sym = wr * (base + 4.5 * cu * cu);
-        const double feq_anti = 3.0 * wr * cu;
-        const double src_sym = pw * (9.0 * cu * cF - 3.0 * uF);
-        const double src_anti = 3.0 * pw * cF;
-        const double sym = m.omega_f * feq_sym + src_sym;
-        const double anti = m.omega_f * feq_anti + src_anti;
-        f[i] = keep * f[i] + (sym + anti);
-        f[i + 1] = keep * f[i + 1] + (sym - anti);
-    }
-    const double feq0 = wgt<double>(0) * rho * base;
-    const double src0 = m.force_pre * wgt<double>(0) * (-3.0 * uF);
-    f[0] = keep * f[0] + (m.omega_f * feq0 + src0);
+    collide_f_pairs<false>(f, rho, ux, uy, uz, Fx, Fy, Fz, m.omega_f, m.pc);
 }
 
 template <>
@@ -535,72 +627,70 @@ __device__ __forceinline__ float add_bf16(float acc, unsigned short bits) {
 //   new- = f- - omega- (f- - feq-) + (1 - omega-/2) S-,
 //   f_i = new+ + new-,  f_{i+1} = new+ - new-.
 // The rest population has only an even part. In FP32 its equilibrium is rho
-// minus the 18 moving ones (as in collide_f), which keeps mass exact.
-template <class R>
-__device__ __forceinline__ void collide_f_trt(R (&f)[Q], R rho, R ux, R uy, R uz, R Fx, R Fy, R Fz,
-                                              const Model<R>& m) {
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R uF = ux * Fx + uy * Fy + uz * Fz;
-    R moving = R(0);
+// minus the 18 moving ones (as in collide_f), which keeps mass exact. FP64
+// runs the pair form shared with BGK.
+__device__ __forceinline__ void collide_f_trt(float (&f)[Q], float rho, float ux, float uy, float uz, float Fx,
+                                              float Fy, float Fz, const Model<float>& m) {
+    const float uu = ux * ux + uy * uy + uz * uz;
+    const float uF = ux * Fx + uy * Fy + uz * Fz;
+    float moving = 0.0f;
 #pragma unroll
     for (int i = 1; i < Q; i += 2) {
-        const R w = wgt<R>(i);
-        const R cu = cdot(i, ux, uy, uz);
-        const R cF = cdot(i, Fx, Fy, Fz);
-        const R ep = w * rho * (R(1) + R(4.5) * cu * cu - R(1.5) * uu);
-        const R em = R(3) * w * rho * cu;
-        const R sp = w * (R(9) * cu * cF - R(3) * uF);
-        const R sm = R(3) * w * cF;
-        const R fp = R(0.5) * (f[i] + f[i + 1]), fm = R(0.5) * (f[i] - f[i + 1]);
-        const R np = fp - m.omega_f * (fp - ep) + m.force_pre * sp;
-        const R nm = fm - m.omega_m * (fm - em) + m.force_pre_m * sm;
+        const float w = wgt<float>(i);
+        const float cu = cdot(i, ux, uy, uz);
+        const float cF = cdot(i, Fx, Fy, Fz);
+        const float ep = w * rho * (1.0f + 4.5f * cu * cu - 1.5f * uu);
+        const float em = 3.0f * w * rho * cu;
+        const float sp = w * (9.0f * cu * cF - 3.0f * uF);
+        const float sm = 3.0f * w * cF;
+        const float fp = 0.5f * (f[i] + f[i + 1]), fm = 0.5f * (f[i] - f[i + 1]);
+        const float np = fp - m.omega_f * (fp - ep) + m.force_pre * sp;
+        const float nm = fm - m.omega_m * (fm - em) + m.force_pre_m * sm;
         f[i] = np + nm;
         f[i + 1] = np - nm;
         moving += ep;
     }
-    const R feq0 = sizeof(R) == 4 ? rho - R(2) * moving : wgt<R>(0) * rho * (R(1) - R(1.5) * uu);
-    const R s0 = wgt<R>(0) * (R(3) * (-uF));
+    const float feq0 = rho - 2.0f * moving;
+    const float s0 = wgt<float>(0) * (3.0f * (-uF));
     f[0] = f[0] - m.omega_f * (f[0] - feq0) + m.force_pre * s0;
 }
-
-// BGK collision of g in place: the generic template direction by direction;
-// FP64 and FP32 on opposite pairs (FP32 with the rest equilibrium phi minus
-// the moving ones, as in collide_f).
-template <class R>
-__device__ __forceinline__ void collide_g(R (&g)[Q], R phi, R mu, R ux, R uy, R uz, const Model<R>& m) {
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R dev = m.Gamma * mu - phi / R(3);
-#pragma unroll
-    for (int i = 1; i < Q; ++i) {
-        const R cu = cdot(i, ux, uy, uz);
-        const R geq = wgt<R>(i) * (phi + R(3) * phi * cu + R(4.5) * dev * R(c2(i) - 1)
-                                   + R(4.5) * phi * cu * cu - R(1.5) * phi * uu);
-        g[i] = g[i] - m.omega_g * (g[i] - geq);
-    }
-    // c_0 = 0, |c_0|^2 - 1 = -1: geq_0 = w_0 (phi - 9/2 dev - 3/2 phi u.u)
-    const R geq0 = wgt<R>(0) * ((phi - R(4.5) * dev) - R(1.5) * phi * uu);
-    g[0] = g[0] - m.omega_g * (g[0] - geq0);
+__device__ __forceinline__ void collide_f_trt(double (&f)[Q], double rho, double ux, double uy, double uz, double Fx,
+                                              double Fy, double Fz, const Model<double>& m) {
+    collide_f_pairs<true>(f, rho, ux, uy, uz, Fx, Fy, Fz, m.omega_f, m.pc);
 }
 
+// BGK collision of g in place, on opposite pairs (FP32 with the rest
+// equilibrium phi minus the moving ones, as in collide_f).
+template <class R>
+__device__ __forceinline__ void collide_g(R (&g)[Q], R phi, R mu, R ux, R uy, R uz, const Model<R>& m);
+
+// FP64: with p = omega_g phi, the even part of a diagonal pair is
+// w p (1 - 3/2 u.u) + 9/2 w omega_g dev + p (c.u)^2 / 8, an axis pair's twice
+// that without dev, and the odd part p c.u / 12; seven instructions a pair.
 template <>
 __device__ __forceinline__ void collide_g<double>(double (&g)[Q], double phi, double mu, double ux, double uy,
                                                   double uz, const Model<double>& m) {
-    const double uu = ux * ux + uy * uy + uz * uz;
-    const double dev = m.Gamma * mu - phi / 3.0;
-    const double pbase = phi * (1.0 - 1.5 * uu);
-    const double keep = 1.0 - m.omega_g;
+    const PairCoef<double>& k = m.pc;
+    const double uu = __fma_rn(ux, ux, __fma_rn(uy, uy, __dmul_rn(uz, uz)));
+    const double p = m.omega_g * phi;
+    const double a = p * __fma_rn(-1.5, uu, 1.0);
+    const double base = wgt<double>(7) * a;
+    const double dev = __fma_rn(k.g_mu, mu, k.g_phi * phi);
+    const double diag = base + dev, p45 = 0.125 * p, p3 = (1.0 / 12.0) * p;
+    auto put = [&](int i, double even, double odd) {
+        g[i] = __fma_rn(k.keep_g, g[i], even + odd);
+        g[i + 1] = __fma_rn(k.keep_g, g[i + 1], even - odd);
+    };
+    g[0] = __fma_rn(wgt<double>(0), a, __fma_rn(-12.0, dev, k.keep_g * g[0]));
+    const double base2 = base + base, p90 = p45 + p45, p6 = p3 + p3;
+    put(1, __fma_rn(p90 * ux, ux, base2), p6 * ux);
+    put(3, __fma_rn(p90 * uy, uy, base2), p6 * uy);
+    put(5, __fma_rn(p90 * uz, uz, base2), p6 * uz);
 #pragma unroll
-    for (int i = 1; i < Q; i += 2) {
-        const double w = wgt<double>(i);
+    for (int i = 7; i < Q; i += 2) {
         const double cu = cdot(i, ux, uy, uz);
-        const double geq_sym = w * (pbase + 4.5 * dev * double(c2(i) - 1) + 4.5 * phi * cu * cu);
-        const double geq_anti = 3.0 * w * phi * cu;
-        const double sym = m.omega_g * geq_sym, anti = m.omega_g * geq_anti;
-        g[i] = keep * g[i] + (sym + anti);
-        g[i + 1] = keep * g[i + 1] + (sym - anti);
+        put(i, __fma_rn(p45 * cu, cu, diag), p3 * cu);
     }
-    const double geq0 = wgt<double>(0) * ((phi - 4.5 * dev) - 1.5 * phi * uu);
-    g[0] = keep * g[0] + m.omega_g * geq0;
 }
 
 template <>

@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kTX * TY, fused_ctas_per_sm<P>())
             } else {
                 const R nb = phis[mid][hy][hx + 1] + phis[mid][hy][hx - 1] + phis[mid][hy + 1][hx]
                            + phis[mid][hy - 1][hx] + phis[hi][hy][hx] + phis[lo][hy][hx];
-                lap = sub_rn(nb, mul_rn(R(6), c));
+                lap = lap7(c, nb);
             }
             if constexpr (kKeepG)
                 mus[slot][my][mx] = chem_potential_lap(dref.Phi + c, lap, m);
@@ -286,13 +286,11 @@ __global__ void __launch_bounds__(kTX * TY, fused_ctas_per_sm<P>())
             guo_velocity(rho, jx, jy, jz, Fx, Fy, Fz, ux, uy, uz);
             collide_f_dev(f, delta, rho, ux, uy, uz, Fx, Fy, Fz, m, dref);
         } else {
-            R rho = R(0), jx = R(0), jy = R(0), jz = R(0);
 #pragma unroll
-            for (int i = 0; i < Q; ++i) {
+            for (int i = 0; i < Q; ++i)
                 f[i] = Prec<P>::decode(kEarlyF ? fpre[i] : (cok ? fs[i * npad + s] : S(0)), refs[i]);
-                rho += f[i];
-                add_c(i, f[i], jx, jy, jz);
-            }
+            R rho, jx, jy, jz;
+            moments_f(f, rho, jx, jy, jz);
             guo_velocity(rho, jx, jy, jz, Fx, Fy, Fz, ux, uy, uz);
             collide_f(f, rho, ux, uy, uz, Fx, Fy, Fz, m);
         }

@@ -220,19 +220,21 @@ __global__ void __launch_bounds__(kRowThreads, rows_blocks_per_sm<P>())
     if (stress) {  // F = -div P
         stress_force_at(m.iso, stress, npad, s, o, Fx, Fy, Fz);
     } else {  // F = -phi grad(mu)
-        R gmx, gmy, gmz;
-        grad_at(m.iso, mu, s, o, gmx, gmy, gmz);
-        Fx = -ph * gmx, Fy = -ph * gmy, Fz = -ph * gmz;
+        if (m.iso) {
+            R gmx, gmy, gmz;
+            grad_at(1, mu, s, o, gmx, gmy, gmz);
+            Fx = -ph * gmx, Fy = -ph * gmy, Fz = -ph * gmz;
+        } else {
+            force_of_diffs(ph, mu[s + oxp] - mu[s + oxm], mu[s + oyp] - mu[s + oym], mu[s + ozp] - mu[s + ozm], Fx, Fy,
+                           Fz);
+        }
     }
 
     R f[Q];
-    R rho = R(0), jx = R(0), jy = R(0), jz = R(0);
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        f[i] = Prec<P>::decode(fr[i], refs[i]);
-        rho += f[i];
-        add_c(i, f[i], jx, jy, jz);
-    }
+    for (int i = 0; i < Q; ++i) f[i] = Prec<P>::decode(fr[i], refs[i]);
+    R rho, jx, jy, jz;
+    moments_f(f, rho, jx, jy, jz);
     R ux, uy, uz;
     guo_velocity(rho, jx, jy, jz, Fx, Fy, Fz, ux, uy, uz);
     if (m.trt)
