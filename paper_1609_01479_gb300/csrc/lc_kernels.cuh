@@ -45,36 +45,44 @@ using ld::wgt;
 
 constexpr int kLcThreads = 128;
 
-// a1 = -A0 (1 - gamma/3), a1n = A0 (1 - gamma/3), a2 = A0 gamma: the bulk
-// coefficients of H and of the free energy density (and the products of
-// them the helpers use, formed once here in FP64).
+// The constants the helpers use, formed once here in FP64 (on the FP64 pipe,
+// which bounds the FP64 step, a product of two constants costs every thread
+// an instruction): a1 = -A0 (1 - gamma/3) and a2 = A0 gamma, the bulk
+// coefficients of H; fe_1 = A0 (1 - gamma/3)/2, fe_3 = -a2/3 and fe_2 = a2/4
+// of the free energy density; kappa and xi in the factors that go with the
+// unscaled central differences (twice the derivative).
 // fm: the fluid's BGK + Guo constants (omega_f = 1/tau_f, force_pre =
 // 1 - 1/(2 tau_f)) for the binary fluid's collision of f, which is the same
 // collision.
 template <class T>
 struct LcModel {
-    T A0, gamma, kappa, Gamma, xi, a1, a1n, a2;
-    T a2_3, half_kappa, two_xi, xi2_3, fe_a1, fe_a2;  // a2/3, kappa/2, 2 xi, 2 xi/3, a1n/2, a2/4
+    T Gamma, a1, a2, kappa;
+    T fe_1, fe_2, fe_3, fe_g;          // fe_g = kappa/8
+    T m_kappa4, m_xi, m_2xi, xi2, m_2xi3;  // -kappa/4, -xi, -2 xi, 2 xi, -2 xi/3
+    T rot_p, rot_m, half_xi, m_xi_tr;  // (xi + 1)/4, (xi - 1)/4, xi/2, -xi
     ld::Model<T> fm;
 };
 template <class T>
 LcModel<T> lc_model_of(const lc_params& p) {
     const double a1n = p.A0 * (1.0 - p.gamma / 3.0);
     LcModel<T> m{};
-    m.A0 = (T)p.A0;
-    m.gamma = (T)p.gamma;
-    m.kappa = (T)p.kappa;
     m.Gamma = (T)p.Gamma;
-    m.xi = (T)p.xi;
     m.a1 = (T)(-a1n);
-    m.a1n = (T)a1n;
     m.a2 = (T)(p.A0 * p.gamma);
-    m.a2_3 = (T)(p.A0 * p.gamma / 3.0);
-    m.half_kappa = (T)(0.5 * p.kappa);
-    m.two_xi = (T)(2.0 * p.xi);
-    m.xi2_3 = (T)(2.0 * p.xi / 3.0);
-    m.fe_a1 = (T)(0.5 * a1n);
-    m.fe_a2 = (T)(0.25 * p.A0 * p.gamma);
+    m.kappa = (T)p.kappa;
+    m.fe_1 = (T)(0.5 * a1n);
+    m.fe_2 = (T)(0.25 * p.A0 * p.gamma);
+    m.fe_3 = (T)(-p.A0 * p.gamma / 3.0);
+    m.fe_g = (T)(0.125 * p.kappa);
+    m.m_kappa4 = (T)(-0.25 * p.kappa);
+    m.m_xi = (T)(-p.xi);
+    m.m_2xi = (T)(-2.0 * p.xi);
+    m.xi2 = (T)(2.0 * p.xi);
+    m.m_2xi3 = (T)(-2.0 * p.xi / 3.0);
+    m.rot_p = (T)(0.25 * (p.xi + 1.0));
+    m.rot_m = (T)(0.25 * (p.xi - 1.0));
+    m.half_xi = (T)(0.5 * p.xi);
+    m.m_xi_tr = (T)(-p.xi);
     m.fm.omega_f = (T)(1.0 / p.tau_f);
     m.fm.force_pre = (T)(1.0 - 0.5 / p.tau_f);
     m.fm.omega_m = m.fm.omega_f;
@@ -90,25 +98,19 @@ struct LcGeom {
 
 // Symmetric tensors are held as their six unique components (xx, xy, xz,
 // yy, yz, zz); the stored Q has five, zz = -xx - yy. sym_a/sym_b give the
-// index pair of component k, sym_w its multiplicity in a full contraction
-// (1 on the diagonal, 2 off it), sym_k the component of (a, b).
+// index pair of component k, sym_k the component of (a, b).
 __device__ __forceinline__ int sym_a(int k) { return k < 3 ? 0 : (k < 5 ? 1 : 2); }
 __device__ __forceinline__ int sym_b(int k) { return k < 3 ? k : (k < 5 ? k - 2 : 2); }
-template <class T>
-__device__ __forceinline__ T sym_w(int k) {
-    return (k == 0 || k == 3 || k == 5) ? T(1) : T(2);
-}
 __device__ __forceinline__ int sym_k(int a, int b) {
     const int lo = a < b ? a : b, hi = a < b ? b : a;
     return lo == 0 ? hi : (lo == 1 ? hi + 2 : 5);
 }
 
-// The six components of Q at element offset s of the [5][npad] store.
+// The five stored components of Q at element offset s of the [5][npad] store.
 template <class T>
-__device__ __forceinline__ void lc_load6(const T* q, long long npad, long long s, T (&v)[6]) {
+__device__ __forceinline__ void lc_load5(const T* q, long long npad, long long s, T (&v)[5]) {
 #pragma unroll
     for (int k = 0; k < 5; ++k) v[k] = q[k * npad + s];
-    v[5] = -v[0] - v[3];
 }
 
 // Arithmetic of the stencil helpers below: T itself (float or double), or
@@ -130,14 +132,12 @@ __device__ __forceinline__ LcF2 operator-(LcF2 a, LcF2 b) {
     return LcF2(*reinterpret_cast<const float2*>(&r));
 }
 __device__ __forceinline__ LcF2& operator+=(LcF2& a, LcF2 b) { return a = a + b; }
-// a * b + c: one fused operation for the pairs, the plain expression for T
-// (contracted in FP32, two roundings in the FP64 unit built without
-// contraction).
+// a * b + c in one fused operation, in every arithmetic (explicit, since the
+// FP64 unit is built without contraction): one rounding, and half the FP64
+// instructions of the sum of products.
 __device__ __forceinline__ LcF2 lc_fma(LcF2 a, LcF2 b, LcF2 c) { return LcF2(__ffma2_rn(a.v, b.v, c.v)); }
-template <class T>
-__device__ __forceinline__ T lc_fma(T a, T b, T c) {
-    return a * b + c;
-}
+__device__ __forceinline__ double lc_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float lc_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 // zz = -xx - yy of a traceless tensor
 __device__ __forceinline__ LcF2 lc_zz(LcF2 xx, LcF2 yy) { return LcF2(-1.0) * xx - yy; }
 template <class T>
@@ -146,47 +146,68 @@ __device__ __forceinline__ T lc_zz(T xx, T yy) {
 }
 
 // Model constants of the stencil helpers in arithmetic A (broadcast to both
-// lanes for LcF2): a1 = -A0 (1 - gamma/3), a2 = A0 gamma, a2_3 = a2/3,
-// kappa, xi, two_xi = 2 xi, xi2_3 = 2 xi/3, fe_a1 = a1n/2 and fe_a2 = a2/4 of
-// the free energy density.
+// lanes for LcF2); see LcModel.
 template <class A>
 struct LcCoef {
-    A a1, a2, a2_3, kappa, half_kappa, xi, two_xi, xi2_3, fe_a1, fe_a2;
+    A a1, m_a2, a2, kappa, fe_1, fe_2, fe_3, fe_g, m_kappa4, m_xi, m_2xi, xi2, m_2xi3;
 };
 template <class A, class T>
 __device__ __forceinline__ LcCoef<A> lc_coef(const LcModel<T>& m) {
     LcCoef<A> c;
     c.a1 = A(m.a1);
+    c.m_a2 = A(-m.a2);
     c.a2 = A(m.a2);
-    c.a2_3 = A(m.a2_3);
     c.kappa = A(m.kappa);
-    c.half_kappa = A(m.half_kappa);
-    c.xi = A(m.xi);
-    c.two_xi = A(m.two_xi);
-    c.xi2_3 = A(m.xi2_3);
-    c.fe_a1 = A(m.fe_a1);
-    c.fe_a2 = A(m.fe_a2);
+    c.fe_1 = A(m.fe_1);
+    c.fe_2 = A(m.fe_2);
+    c.fe_3 = A(m.fe_3);
+    c.fe_g = A(m.fe_g);
+    c.m_kappa4 = A(m.m_kappa4);
+    c.m_xi = A(m.m_xi);
+    c.m_2xi = A(m.m_2xi);
+    c.xi2 = A(m.xi2);
+    c.m_2xi3 = A(m.m_2xi3);
     return c;
 }
 
-// Central-difference gradient dQ[c][k] = d_c Q_k and 7-point Laplacian of
-// Q at a site. nb(c, sgn, v) fills v with the six components of the
-// neighbour at sgn * e_c.
+// zz of a traceless tensor into its sixth component.
+template <class A>
+__device__ __forceinline__ void lc_close(A (&v)[6]) {
+    v[5] = lc_zz(v[0], v[3]);
+}
+
+// Unscaled central differences d[c][k] = Q_k(x + e_c) - Q_k(x - e_c) (twice
+// the derivative) and the 7-point Laplacian of the five stored components.
+// nb(c, sgn, v) fills v with the components of the neighbour at sgn * e_c.
 template <class A, class Nb>
-__device__ __forceinline__ void lc_grad_lap(const A (&q)[6], Nb nb, A (&dQ)[3][6], A (&lap)[6]) {
-#pragma unroll
-    for (int k = 0; k < 6; ++k) lap[k] = A(-6.0) * q[k];
+__device__ __forceinline__ void lc_lap(const A (&q)[6], Nb nb, A (&lap)[5]) {
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        A qp[6], qm[6];
+        A qp[5], qm[5];
         nb(c, 1, qp);
         nb(c, -1, qm);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            dQ[c][k] = A(0.5) * (qp[k] - qm[k]);
-            lap[k] += qp[k] + qm[k];
-        }
+        for (int k = 0; k < 5; ++k) lap[k] = c == 0 ? qp[k] + qm[k] : lap[k] + (qp[k] + qm[k]);
     }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lap[k] = lc_fma(A(-6.0), q[k], lap[k]);
+}
+template <class A, class Nb>
+__device__ __forceinline__ void lc_diffs_lap(const A (&q)[6], Nb nb, A (&d)[3][6], A (&lap)[5]) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        A qp[5], qm[5];
+        nb(c, 1, qp);
+        nb(c, -1, qm);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            d[c][k] = qp[k] - qm[k];
+            lap[k] = c == 0 ? qp[k] + qm[k] : lap[k] + (qp[k] + qm[k]);
+        }
+        lc_close(d[c]);
+    }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) lap[k] = lc_fma(A(-6.0), q[k], lap[k]);
 }
 
 // The contraction X:Y of two symmetric tensors from their six components
@@ -195,71 +216,86 @@ template <class A>
 __device__ __forceinline__ A lc_sym_dot(const A (&x)[6], const A (&y)[6]) {
     const A diag = lc_fma(x[5], y[5], lc_fma(x[3], y[3], x[0] * y[0]));
     const A off = lc_fma(x[4], y[4], lc_fma(x[2], y[2], x[1] * y[1]));
-    return diag + (off + off);
+    return lc_fma(A(2.0), off, diag);
+}
+
+// Component k of the square Q.Q (symmetric).
+template <class A>
+__device__ __forceinline__ A lc_square(const A (&q)[6], int k) {
+    const int a = sym_a(k), b = sym_b(k);
+    return lc_fma(q[sym_k(a, 2)], q[sym_k(2, b)],
+                  lc_fma(q[sym_k(a, 1)], q[sym_k(1, b)], q[sym_k(a, 0)] * q[sym_k(0, b)]));
 }
 
 // Molecular field H = -dF/dQ of the Landau-de Gennes free energy with one
-// elastic constant, on the six components:
-//   H = a1 Q + a2 (QQ - tr2 I/3) - a2 tr2 Q + kappa lap Q;
-// also returns tr2 = Q:Q and the square QQ = Q.Q (symmetric) for the stress.
+// elastic constant: H = a1 Q + a2 (QQ - tr2 I/3) - a2 tr2 Q + kappa lap Q.
+// Five components (H is traceless); also returns tr2 = Q:Q and, for the
+// stress, the same five components of QQ.
 template <class A>
-__device__ __forceinline__ void lc_molecular_field(const A (&q)[6], const A (&lap)[6], const LcCoef<A>& m, A& tr2,
+__device__ __forceinline__ void lc_molecular_field(const A (&q)[6], const A (&lap)[5], const LcCoef<A>& m, A& tr2,
                                                    A (&qq)[6], A (&H)[6]) {
     tr2 = lc_sym_dot(q, q);
-    const A tr2_3 = tr2 * A(1.0 / 3.0), a2tr2 = m.a2 * tr2;
+    const A tr2_3 = tr2 * A(1.0 / 3.0), lin = lc_fma(m.m_a2, tr2, m.a1);
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int a = sym_a(k), b = sym_b(k);
-        A s = q[sym_k(a, 0)] * q[sym_k(0, b)];
-        s = lc_fma(q[sym_k(a, 1)], q[sym_k(1, b)], s);
-        s = lc_fma(q[sym_k(a, 2)], q[sym_k(2, b)], s);
-        qq[k] = s;
-        const A dev = a == b ? s - tr2_3 : s;
-        H[k] = lc_fma(m.kappa, lap[k], lc_fma(m.a2, dev, (m.a1 - a2tr2) * q[k]));
+    for (int k = 0; k < 5; ++k) {
+        qq[k] = lc_square(q, k);
+        const A dev = sym_a(k) == sym_b(k) ? qq[k] - tr2_3 : qq[k];
+        H[k] = lc_fma(m.kappa, lap[k], lc_fma(m.a2, dev, lin * q[k]));
     }
 }
 
-// Chemical stress sigma_ab of a site. With P = Q.H (so H.Q = P^T, Q and H
-// being symmetric) the terms of H collapse to
+// Chemical stress sigma_ab of a site from Q, its unscaled differences d, H
+// and QQ (zz of both filled in here), tr2. With P = Q.H (so H.Q = P^T, Q and
+// H being symmetric) the terms of H collapse to
 //   -xi (P_ab + P_ba) - (2 xi/3) H_ab + 2 xi (Q_ab + delta_ab/3) Q:H + P_ab - P_ba,
-// the elastic term is -kappa G_ab with G_ab = d_a Q_cd d_b Q_cd (symmetric),
-// and the free energy density f on the diagonal uses |grad Q|^2 = tr G and
-// tr(Q^3) = QQ:Q. out(a, b, value) receives each component.
+// the elastic term is -kappa G_ab with 4 G_ab = d_a Q_cd d_b Q_cd of the
+// unscaled differences (symmetric), and the free energy density f on the
+// diagonal uses |grad Q|^2 = tr G and tr(Q^3) = QQ:Q. The two components of
+// an off-diagonal pair share all but the sign of P_ab - P_ba. out(a, b, value)
+// receives each component. About 170 operations; the FP64 field launch ran
+// 383 FP64 instructions a site when the six components of every neighbour,
+// scaled derivatives and each of the nine sigma_ab were formed separately
+// with unfused products.
 template <class A, class Out>
-__device__ __forceinline__ void lc_stress(const A (&q)[6], const A (&dQ)[3][6], const A (&H)[6], const A (&qq)[6],
-                                          A tr2, const LcCoef<A>& m, Out out) {
+__device__ __forceinline__ void lc_stress(const A (&q)[6], const A (&d)[3][6], A (&H)[6], A (&qq)[6], A tr2,
+                                          const LcCoef<A>& m, Out out) {
+    lc_close(H);
+    qq[5] = lc_square(q, 5);
     const A tr3 = lc_sym_dot(qq, q), qh = lc_sym_dot(q, H);
     A G[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-        const int a = sym_a(k), b = sym_b(k);
-        const A diag = lc_fma(dQ[a][5], dQ[b][5], lc_fma(dQ[a][3], dQ[b][3], dQ[a][0] * dQ[b][0]));
-        const A off = lc_fma(dQ[a][4], dQ[b][4], lc_fma(dQ[a][2], dQ[b][2], dQ[a][1] * dQ[b][1]));
-        G[k] = diag + (off + off);
-    }
-    const A grad2 = G[0] + G[3] + G[5];
+    for (int k = 0; k < 6; ++k) G[k] = lc_sym_dot(d[sym_a(k)], d[sym_b(k)]);
     // f = a1n/2 tr2 - a2/3 tr3 + a2/4 tr2^2 + kappa/2 |grad Q|^2
-    const A fe = lc_fma(m.half_kappa, grad2, lc_fma(m.fe_a2 * tr2, tr2, m.fe_a1 * tr2 - m.a2_3 * tr3));
+    const A fe = lc_fma(m.fe_g, G[0] + G[3] + G[5], lc_fma(m.fe_3, tr3, lc_fma(m.fe_2, tr2, m.fe_1) * tr2));
     A P[3][3];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            A s = q[sym_k(a, 0)] * H[sym_k(0, b)];
-            s = lc_fma(q[sym_k(a, 1)], H[sym_k(1, b)], s);
-            P[a][b] = lc_fma(q[sym_k(a, 2)], H[sym_k(2, b)], s);
-        }
-    const A tq = m.two_xi * qh;
+        for (int b = 0; b < 3; ++b)
+            P[a][b] = lc_fma(q[sym_k(a, 2)], H[sym_k(2, b)],
+                             lc_fma(q[sym_k(a, 1)], H[sym_k(1, b)], q[sym_k(a, 0)] * H[sym_k(0, b)]));
+    const A tq = m.xi2 * qh, iso = lc_fma(tq, A(1.0 / 3.0), fe);
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int a = 0; a < 3; ++a) {
+        const int k = sym_k(a, a);
+        const A v = lc_fma(m.m_2xi3, H[k], lc_fma(m.m_kappa4, G[k], lc_fma(m.m_2xi, P[a][a], iso)));
+        out(a, a, lc_fma(tq, q[k], v));
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            const int k = sym_k(a, b);
-            // 2 xi (Q + delta/3) Q:H - (2 xi/3) H - kappa G - xi (P + P^T) + (P - P^T) [+ f]
-            A v = lc_fma(tq, a == b ? q[k] + A(1.0 / 3.0) : q[k], (P[a][b] - P[b][a]) - m.xi * (P[a][b] + P[b][a]));
-            v = v - lc_fma(m.kappa, G[k], m.xi2_3 * H[k]);
-            out(a, b, a == b ? v + fe : v);
+        for (int b = a + 1; b < 3; ++b) {
+            const int o = sym_k(a, b);
+            const A even = lc_fma(tq, q[o], lc_fma(m.m_xi, P[a][b] + P[b][a], lc_fma(m.m_kappa4, G[o], m.m_2xi3 * H[o])));
+            const A odd = P[a][b] - P[b][a];
+            out(a, b, even + odd);
+            out(b, a, even - odd);
         }
+    }
+}
+
+// F_a = d_b sigma_ab from the unscaled differences of sigma_a0, sigma_a1 and
+// sigma_a2 along x, y and z.
+template <class T>
+__device__ __forceinline__ T lc_force(T dx, T dy, T dz) {
+    return T(0.5) * ((dx + dy) + dz);
 }
 
 // Velocity u = (j + F/2)/rho and the BGK + Guo collision of one site's f
@@ -280,38 +316,49 @@ __device__ __forceinline__ void lc_collide_site(T (&fv)[Q], const T (&Fa)[3], co
 }
 
 // The Q update of one site: Q + Gamma H + S(W, Q) - u.grad(Q), the
-// advection first-order upwind, W_ab = d_b u_a from the central difference
-// of u. qnb(k, c, sgn) is component k of Q at the neighbour sgn * e_c.
+// advection first-order upwind, W_ab = d_b u_a from the unscaled central
+// differences dU_ab = 2 W_ab of u. With M = xi D + Om, whose transpose is
+// xi D - Om, and the symmetric Q' = Q + I/3, the co-rotation is
+//   S = M Q' + (M Q')^T - 2 xi Q' tr(Q W),
+// M_ab = (xi + 1)/4 dU_ab + (xi - 1)/4 dU_ba. The increment is summed apart
+// from Q, which is added last. qnb(k, c, sgn) is component k of Q at the
+// neighbour sgn * e_c. 115 operations (259 FP64 instructions with D, Om and
+// both products formed separately, unfused).
 template <class T, class QNb>
-__device__ __forceinline__ void lc_update_site(const T (&q)[6], const T (&H)[6], const T (&us)[3], const T (&W)[3][3],
+__device__ __forceinline__ void lc_update_site(const T (&q)[6], const T (&H)[6], const T (&us)[3], const T (&dU)[3][3],
                                                const LcModel<T>& m, QNb qnb, T (&qn)[5]) {
-    T D[3][3], Om[3][3], Qp[3][3];
-    T trQW = T(0);
+    T M[3][3], Qp[6];
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            D[a][b] = T(0.5) * (W[a][b] + W[b][a]);
-            Om[a][b] = T(0.5) * (W[a][b] - W[b][a]);
-            Qp[a][b] = q[sym_k(a, b)] + (a == b ? T(1) / T(3) : T(0));
-            trQW += q[sym_k(a, b)] * W[b][a];
-        }
+        for (int b = 0; b < 3; ++b)
+            M[a][b] = a == b ? m.half_xi * dU[a][a] : lc_fma(m.rot_p, dU[a][b], m.rot_m * dU[b][a]);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) Qp[k] = sym_a(k) == sym_b(k) ? q[k] + T(1.0 / 3.0) : q[k];
+    T tr = lc_fma(q[5], dU[2][2], lc_fma(q[3], dU[1][1], q[0] * dU[0][0]));  // 2 tr(Q W)
+    tr = lc_fma(q[1], dU[0][1] + dU[1][0], tr);
+    tr = lc_fma(q[2], dU[0][2] + dU[2][0], tr);
+    tr = lc_fma(q[4], dU[1][2] + dU[2][1], tr);
+    const T tw = m.m_xi_tr * tr;  // -2 xi tr(Q W)
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
         const int a = sym_a(k), b = sym_b(k);
-        T S = T(0);
+        T S = lc_fma(M[a][2], Qp[sym_k(2, b)], lc_fma(M[a][1], Qp[sym_k(1, b)], M[a][0] * Qp[sym_k(0, b)]));
+        if (a == b) {
+            S = S + S;
+        } else {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) S += (m.xi * D[a][c] + Om[a][c]) * Qp[c][b] + Qp[a][c] * (m.xi * D[c][b] - Om[c][b]);
-        S = S - T(2) * m.xi * Qp[a][b] * trQW;
+            for (int c = 0; c < 3; ++c) S = lc_fma(M[b][c], Qp[sym_k(c, a)], S);
+        }
+        S = lc_fma(m.Gamma, H[k], lc_fma(tw, Qp[k], S));
         const T qc = q[k];
-        T adv = T(0);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const bool fwd = us[c] >= T(0);
-            const T diff = fwd ? qc - qnb(k, c, -1) : qnb(k, c, 1) - qc;
-            adv += us[c] * diff;
+            const T hi = fwd ? qc : qnb(k, c, 1), lo = fwd ? qnb(k, c, -1) : qc;
+            S = lc_fma(-us[c], hi - lo, S);
         }
-        qn[k] = qc + m.Gamma * H[k] + S - adv;
+        qn[k] = qc + S;
     }
 }
 
@@ -340,15 +387,29 @@ __device__ __forceinline__ bool lc_site_of(const LcGeom& g, LcSite& t) {
 }
 __device__ __forceinline__ int lc_nb(const LcSite& t, int c, int sgn) { return t.nbr[2 * c + (sgn > 0 ? 0 : 1)]; }
 
+// F_a at a site from the stored sigma [9][npad].
+template <class T>
+__device__ __forceinline__ T lc_force_at(const LcGeom& g, const LcSite& t, const T* sigma, int a) {
+    T d[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const T* sg = sigma + (3 * a + b) * g.npad;
+        d[b] = sg[lc_nb(t, b, 1)] - sg[lc_nb(t, b, -1)];
+    }
+    return lc_force(d[0], d[1], d[2]);
+}
+
 template <class T>
 __global__ void __launch_bounds__(kLcThreads) k_lc_field(LcGeom g, LcModel<T> m, const T* __restrict__ q,
                                                          T* __restrict__ h, T* __restrict__ sigma) {
     LcSite t;
     if (!lc_site_of(g, t)) return;
     const LcCoef<T> cf = lc_coef<T>(m);
-    T q6[6], dQ[3][6], lap[6], H[6], qq[6], tr2;
-    lc_load6(q, g.npad, t.s, q6);
-    lc_grad_lap(q6, [&](int c, int sgn, T (&v)[6]) { lc_load6(q, g.npad, lc_nb(t, c, sgn), v); }, dQ, lap);
+    T q6[6], dQ[3][6], lap[5], H[6], qq[6], tr2;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) q6[k] = q[k * g.npad + t.s];
+    lc_close(q6);
+    lc_diffs_lap(q6, [&](int c, int sgn, T (&v)[5]) { lc_load5(q, g.npad, lc_nb(t, c, sgn), v); }, dQ, lap);
     lc_molecular_field(q6, lap, cf, tr2, qq, H);
     lc_stress(q6, dQ, H, qq, tr2, cf, [&](int a, int b, T v) { sigma[(3 * a + b) * g.npad + t.s] = v; });
 #pragma unroll
@@ -361,13 +422,9 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_collide(LcGeom g, LcModel<T> 
                                                            T* __restrict__ u) {
     LcSite t;
     if (!lc_site_of(g, t)) return;
-    T Fa[3] = {T(0), T(0), T(0)};
+    T Fa[3];
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        const int sp = lc_nb(t, b, 1), sm = lc_nb(t, b, -1);
-#pragma unroll
-        for (int a = 0; a < 3; ++a) Fa[a] += T(0.5) * (sigma[(3 * a + b) * g.npad + sp] - sigma[(3 * a + b) * g.npad + sm]);
-    }
+    for (int a = 0; a < 3; ++a) Fa[a] = lc_force_at(g, t, sigma, a);
     T fv[Q], uv[3];
 #pragma unroll
     for (int i = 0; i < Q; ++i) fv[i] = f[i * g.npad + t.s];
@@ -392,35 +449,36 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_update(LcGeom g, LcModel<T> m
                                                           T* __restrict__ qn) {
     LcSite t;
     if (!lc_site_of(g, t)) return;
-    T W[3][3], q6[6], H[6], us[3], qv[5];
+    T dU[3][3], q6[6], H[6], us[3], qv[5];
 #pragma unroll
     for (int a = 0; a < 3; ++a) us[a] = u[a * g.npad + t.s];
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
         const int sp = lc_nb(t, b, 1), sm = lc_nb(t, b, -1);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) W[a][b] = T(0.5) * (u[a * g.npad + sp] - u[a * g.npad + sm]);
+        for (int a = 0; a < 3; ++a) dU[a][b] = u[a * g.npad + sp] - u[a * g.npad + sm];
     }
-    lc_load6(q, g.npad, t.s, q6);
-    T qnb[3][2][6];  // Q at the six neighbours, for H and the upwind differences
+#pragma unroll
+    for (int k = 0; k < 5; ++k) q6[k] = q[k * g.npad + t.s];
+    lc_close(q6);
+    T qnb[3][2][5];  // Q at the six neighbours, for H and the upwind differences
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        lc_load6(q, g.npad, lc_nb(t, c, 1), qnb[c][0]);
-        lc_load6(q, g.npad, lc_nb(t, c, -1), qnb[c][1]);
+        lc_load5(q, g.npad, lc_nb(t, c, 1), qnb[c][0]);
+        lc_load5(q, g.npad, lc_nb(t, c, -1), qnb[c][1]);
     }
     if constexpr (RECOMPUTE_H) {
-        T dQ[3][6], lap[6], qq[6], tr2;
-        lc_grad_lap(q6, [&](int c, int sgn, T (&v)[6]) {
+        T lap[5], qq[6], tr2;
+        lc_lap(q6, [&](int c, int sgn, T (&v)[5]) {
 #pragma unroll
-            for (int k = 0; k < 6; ++k) v[k] = qnb[c][sgn > 0 ? 0 : 1][k];
-        }, dQ, lap);
+            for (int k = 0; k < 5; ++k) v[k] = qnb[c][sgn > 0 ? 0 : 1][k];
+        }, lap);
         lc_molecular_field(q6, lap, lc_coef<T>(m), tr2, qq, H);
     } else {
 #pragma unroll
         for (int k = 0; k < 5; ++k) H[k] = h[k * g.npad + t.s];
-        H[5] = T(0);  // unused by the update
     }
-    lc_update_site(q6, H, us, W, m, [&](int k, int c, int sgn) { return qnb[c][sgn > 0 ? 0 : 1][k]; }, qv);
+    lc_update_site(q6, H, us, dU, m, [&](int k, int c, int sgn) { return qnb[c][sgn > 0 ? 0 : 1][k]; }, qv);
 #pragma unroll
     for (int k = 0; k < 5; ++k) qn[k * g.npad + t.s] = qv[k];
 }
@@ -441,7 +499,7 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_update(LcGeom g, LcModel<T> m
 // f(k) from shared memory and store f and u. Per site the launch reads Q once
 // from HBM (halo re-reads hit L2) and f once, and writes f and u; H and sigma
 // never leave the SM. The arithmetic of every site is the per-site kernels'
-// (lc_grad_lap, lc_molecular_field, lc_stress, lc_collide_site), in the same
+// (lc_diffs_lap, lc_molecular_field, lc_stress, lc_collide_site), in the same
 // order, so FP64 gives their bits.
 constexpr int kLcTX = 32, kLcTY = 8, kLcFusedThreads = kLcTX * kLcTY;
 constexpr int kLcQW = kLcTX + 4, kLcQH = kLcTY + 4;  // Q ring plane (tile + 2-halo)
@@ -541,11 +599,6 @@ __global__ void __launch_bounds__(kLcFusedThreads, (lc_fused_ctas<T, STAGE_F>())
             lc_cp_async<16>(&FT(i, r, c), f + i * npad + (zp * plane + (y0 + r) * nx + x0 + c));
         }
     };
-    auto six_at = [&](int slot, int py, int px, T (&v)[6]) {
-#pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = QR(slot, k, py, px);
-        v[5] = -v[0] - v[3];
-    };
     // The sigma components that F reads, of the site at (hx, hy) of the
     // tile + 1-halo frame: sigma_a0 on the tile rows, sigma_a1 on the tile
     // columns, sigma_a2 on the tile; into slot xy of SX/SY and zs of SZ.
@@ -567,15 +620,17 @@ __global__ void __launch_bounds__(kLcFusedThreads, (lc_fused_ctas<T, STAGE_F>())
             for (int idx = tid; idx < kPairsX * (kLcTY + 2); idx += kLcFusedThreads) {
                 const int hx = 2 * (idx % kPairsX), hy = idx / kPairsX;
                 const int px = hx + 1, py = hy + 1;
-                auto six2 = [&](int slot, int yy, int xx, LcF2 (&v)[6]) {
-#pragma unroll
-                    for (int k = 0; k < 5; ++k) v[k] = LcF2(make_float2(QR(slot, k, yy, xx), QR(slot, k, yy, xx + 1)));
-                    v[5] = lc_zz(v[0], v[3]);
+                auto at = [&](int slot, int k, int yy, int xx) {
+                    return LcF2(make_float2(QR(slot, k, yy, xx), QR(slot, k, yy, xx + 1)));
                 };
-                LcF2 q6[6], dQ[3][6], lap[6], H[6], qq[6], tr2;
-                six2(mid, py, px, q6);
-                lc_grad_lap(q6, [&](int c, int sgn, LcF2 (&v)[6]) {
-                    six2(c == 2 ? (sgn > 0 ? hi : lo) : mid, py + sgn * (c == 1), px + sgn * (c == 0), v);
+                LcF2 q6[6], dQ[3][6], lap[5], H[6], qq[6], tr2;
+#pragma unroll
+                for (int k = 0; k < 5; ++k) q6[k] = at(mid, k, py, px);
+                lc_close(q6);
+                lc_diffs_lap(q6, [&](int c, int sgn, LcF2 (&v)[5]) {
+#pragma unroll
+                    for (int k = 0; k < 5; ++k)
+                        v[k] = at(c == 2 ? (sgn > 0 ? hi : lo) : mid, k, py + sgn * (c == 1), px + sgn * (c == 0));
                 }, dQ, lap);
                 lc_molecular_field(q6, lap, cf, tr2, qq, H);
                 lc_stress(q6, dQ, H, qq, tr2, cf, [&](int a, int b, LcF2 v) {
@@ -600,10 +655,14 @@ __global__ void __launch_bounds__(kLcFusedThreads, (lc_fused_ctas<T, STAGE_F>())
                     hy = (j / kLcTX) * (kLcTY + 1);
                 }
                 const int px = hx + 1, py = hy + 1;
-                T q6[6], dQ[3][6], lap[6], H[6], qq[6], tr2;
-                six_at(mid, py, px, q6);
-                lc_grad_lap(q6, [&](int c, int sgn, T (&v)[6]) {
-                    six_at(c == 2 ? (sgn > 0 ? hi : lo) : mid, py + sgn * (c == 1), px + sgn * (c == 0), v);
+                T q6[6], dQ[3][6], lap[5], H[6], qq[6], tr2;
+#pragma unroll
+                for (int k = 0; k < 5; ++k) q6[k] = QR(mid, k, py, px);
+                lc_close(q6);
+                lc_diffs_lap(q6, [&](int c, int sgn, T (&v)[5]) {
+#pragma unroll
+                    for (int k = 0; k < 5; ++k)
+                        v[k] = QR(c == 2 ? (sgn > 0 ? hi : lo) : mid, k, py + sgn * (c == 1), px + sgn * (c == 0));
                 }, dQ, lap);
                 lc_molecular_field(q6, lap, cf, tr2, qq, H);
                 lc_stress(q6, dQ, H, qq, tr2, cf, [&](int a, int b, T v) { put_sigma(hx, hy, xy, zs, a, b, v); });
@@ -644,14 +703,12 @@ __global__ void __launch_bounds__(kLcFusedThreads, (lc_fused_ctas<T, STAGE_F>())
         __syncthreads();
 
         const int s = k * plane + y * nx + x;  // z1 <= nz
-        T Fa[3] = {T(0), T(0), T(0)};
+        T Fa[3];
         const int sxy = xs(k), szp = ss(k + 1), szm = ss(k - 1);
 #pragma unroll
-        for (int a = 0; a < 3; ++a) Fa[a] += T(0.5) * (SX(sxy, a, ty, tx + 2) - SX(sxy, a, ty, tx));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) Fa[a] += T(0.5) * (SY(sxy, a, ty + 2, tx) - SY(sxy, a, ty, tx));
-#pragma unroll
-        for (int a = 0; a < 3; ++a) Fa[a] += T(0.5) * (SZ(szp, a, ty, tx) - SZ(szm, a, ty, tx));
+        for (int a = 0; a < 3; ++a)
+            Fa[a] = lc_force(SX(sxy, a, ty, tx + 2) - SX(sxy, a, ty, tx), SY(sxy, a, ty + 2, tx) - SY(sxy, a, ty, tx),
+                             SZ(szp, a, ty, tx) - SZ(szm, a, ty, tx));
         T fv[Q], uv[3];
 #pragma unroll
         for (int i = 0; i < Q; ++i) fv[i] = STAGE_F ? FT(i, ty, tx) : __ldcs(f + i * npad + s);
@@ -724,12 +781,8 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_out(LcGeom g, const T* __rest
     if (fo)
         for (int i = 0; i < Q; ++i) fo[i * g.n + s] = (double)f[i * g.npad + s];
     if (rho || uo) {
-        T Fa[3] = {T(0), T(0), T(0)};
-        for (int b = 0; b < 3; ++b) {
-            const int sp = lc_nb(t, b, 1), sm = lc_nb(t, b, -1);
-            for (int a = 0; a < 3; ++a)
-                Fa[a] += T(0.5) * (sigma[(3 * a + b) * g.npad + sp] - sigma[(3 * a + b) * g.npad + sm]);
-        }
+        T Fa[3];
+        for (int a = 0; a < 3; ++a) Fa[a] = lc_force_at(g, t, sigma, a);
         T fv[Q], r, uv[3];
 #pragma unroll
         for (int i = 0; i < Q; ++i) fv[i] = f[i * g.npad + s];
