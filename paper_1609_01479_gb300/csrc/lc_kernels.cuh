@@ -753,12 +753,7 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_init(LcGeom g, double rho0, c
     if (s >= g.n) return;
     const T r = rho ? (T)rho[s] : (T)rho0;
     const T ux = uin ? (T)uin[s] : T(0), uy = uin ? (T)uin[g.n + s] : T(0), uz = uin ? (T)uin[2 * g.n + s] : T(0);
-    const T uu = ux * ux + uy * uy + uz * uz;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const T cu = T(cx(i)) * ux + T(cy(i)) * uy + T(cz(i)) * uz;
-        f[i * g.npad + s] = wgt<T>(i) * r * (T(1) + T(3) * cu + T(4.5) * cu * cu - T(1.5) * uu);
-    }
+    ld::equilibria(r, T(0), T(0), T(0), ux, uy, uz, [&](int i, T feq, T) { f[i * g.npad + s] = feq; });
 #pragma unroll
     for (int k = 0; k < 5; ++k) q[k * g.npad + s] = (T)qin[k * g.n + s];
 }

@@ -37,10 +37,28 @@ __host__ __device__ constexpr R wgt(int i) {
 }
 
 // ---------------------------------------------------------------------------
+// x - y rounded to odd (Boldo & Melquiond 2008): the difference truncated
+// toward zero, with the last bit set where it is inexact. Rounding the
+// result to a format of at most 22 bits gives what rounding the exact
+// difference once would. The error of the float difference is exact (Knuth's
+// two-sum); truncated with the sticky bit, an inexact difference whose last
+// bit is clear moves by one unit, away from zero if the error has its sign,
+// else toward zero. Eight FP32 and integer operations instead of two
+// conversions and a subtraction on the FP64 pipe.
+__device__ __forceinline__ float sub_to_odd(float x, float y) {
+    const float d = __fsub_rn(x, y);
+    const float b = __fsub_rn(d, x);
+    const float e = __fsub_rn(__fsub_rn(x, __fsub_rn(d, b)), __fadd_rn(y, b));
+    const int u = __float_as_int(d), v = __float_as_int(e);
+    if (e == 0.0f || (u & 1) || !(fabsf(d) <= 3.4028234e38f)) return d;
+    return __int_as_float((u ^ v) < 0 ? u - 1 : u + 1);
+}
+
 // Storage precisions. real_t is the arithmetic type; store_t the stored one.
 // The 16-bit forms store the deviation from a per-direction reference value.
 // decode/encode work in real_t inside the step; decode_d/encode_d convert
-// to and from double for initialisation, I/O and the FP64 totals.
+// to and from double for I/O and the FP64 totals; encode_r rounds a real_t
+// value less its reference once, to the bits that encode_d gives for it.
 template <int P> struct Prec;
 template <> struct Prec<LD_FP64> {
     using store_t = double;
@@ -50,6 +68,7 @@ template <> struct Prec<LD_FP64> {
     __device__ static store_t encode(double x, double) { return x; }
     __device__ static double decode_d(store_t v, float) { return v; }
     __device__ static store_t encode_d(double x, float) { return x; }
+    __device__ static store_t encode_r(double x, float) { return x; }
 };
 template <> struct Prec<LD_FP32> {
     using store_t = float;
@@ -59,6 +78,7 @@ template <> struct Prec<LD_FP32> {
     __device__ static store_t encode(float x, float) { return x; }
     __device__ static double decode_d(store_t v, float) { return v; }
     __device__ static store_t encode_d(double x, float) { return (float)x; }
+    __device__ static store_t encode_r(float x, float) { return x; }
 };
 template <> struct Prec<LD_FP16DEV> {
     using store_t = __half;
@@ -69,6 +89,7 @@ template <> struct Prec<LD_FP16DEV> {
     __device__ static store_t encode_sr(float x, float ref, unsigned k);
     __device__ static double decode_d(store_t v, float ref) { return (double)ref + (double)__half2float(v); }
     __device__ static store_t encode_d(double x, float ref) { return __double2half(x - (double)ref); }
+    __device__ static store_t encode_r(float x, float ref) { return __float2half_rn(sub_to_odd(x, ref)); }
 };
 template <> struct Prec<LD_BF16DEV> {
     using store_t = __nv_bfloat16;
@@ -79,6 +100,7 @@ template <> struct Prec<LD_BF16DEV> {
     __device__ static store_t encode_sr(float x, float ref, unsigned k);
     __device__ static double decode_d(store_t v, float ref) { return (double)ref + (double)__bfloat162float(v); }
     __device__ static store_t encode_d(double x, float ref) { return __double2bfloat16(x - (double)ref); }
+    __device__ static store_t encode_r(float x, float ref) { return __float2bfloat16_rn(sub_to_odd(x, ref)); }
 };
 
 // Stochastic rounding of the FP32 deviation h to a 16-bit format with the
@@ -657,6 +679,42 @@ __device__ __forceinline__ void collide_f_trt(float (&f)[Q], float rho, float ux
 __device__ __forceinline__ void collide_f_trt(double (&f)[Q], double rho, double ux, double uy, double uz, double Fx,
                                               double Fy, double Fz, const Model<double>& m) {
     collide_f_pairs<true>(f, rho, ux, uy, uz, Fx, Fy, Fz, m.omega_f, m.pc);
+}
+
+// Equilibria of a site, feq_i and geq_i, handed to out(i, feq, geq): one
+// direction at a time in FP32; on opposite pairs with fused operations in FP64,
+// where 19 directions took about 330 instructions on the FP64 pipe.
+template <class Out>
+__device__ __forceinline__ void equilibria(float rho, float p, float mu, float Gamma, float ux, float uy, float uz,
+                                           Out out) {
+    const float uu = ux * ux + uy * uy + uz * uz;
+    const float dev = Gamma * mu - p / 3.0f;
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+        const float cu = cdot(i, ux, uy, uz);
+        const float feq = wgt<float>(i) * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * uu);
+        const float geq = wgt<float>(i) * (p + 3.0f * p * cu + 4.5f * dev * float(c2(i) - 1) + 4.5f * p * cu * cu -
+                                           1.5f * p * uu);
+        out(i, feq, geq);
+    }
+}
+template <class Out>
+__device__ __forceinline__ void equilibria(double rho, double p, double mu, double Gamma, double ux, double uy,
+                                           double uz, Out out) {
+    const double uu = __fma_rn(ux, ux, __fma_rn(uy, uy, __dmul_rn(uz, uz)));
+    const double base = __fma_rn(-1.5, uu, 1.0);
+    const double dev45 = 4.5 * __fma_rn(Gamma, mu, (-1.0 / 3.0) * p);
+    const double rb = rho * base, pb = p * base;
+    out(0, wgt<double>(0) * rb, wgt<double>(0) * (pb - dev45));
+#pragma unroll
+    for (int i = 1; i < Q; i += 2) {
+        const double w = wgt<double>(i), cu = cdot(i, ux, uy, uz);
+        const double even = __fma_rn(4.5 * cu, cu, base), odd = 3.0 * cu;
+        const double wr = w * rho, wp = w * p;
+        const double fe = wr * even, ge = c2(i) == 2 ? __fma_rn(wp, even, w * dev45) : wp * even;
+        out(i, __fma_rn(wr, odd, fe), __fma_rn(wp, odd, ge));
+        out(i + 1, __fma_rn(-wr, odd, fe), __fma_rn(-wp, odd, ge));
+    }
 }
 
 // BGK collision of g in place, on opposite pairs (FP32 with the rest

@@ -306,17 +306,10 @@ __global__ void __launch_bounds__(kThreads)
         uy = (R)u_in[g.n + s];
         uz = (R)u_in[2 * g.n + s];
     }
-    const R uu = ux * ux + uy * uy + uz * uz;
-    const R dev = m.Gamma * mu - p / R(3);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const R cu = cdot(i, ux, uy, uz);
-        const R feq = wgt<R>(i) * rho * (R(1) + R(3) * cu + R(4.5) * cu * cu - R(1.5) * uu);
-        const R geq = wgt<R>(i) * (p + R(3) * p * cu + R(4.5) * dev * R(c2(i) - 1) + R(4.5) * p * cu * cu
-                                   - R(1.5) * p * uu);
-        fd[i * g.npad + s] = Prec<P>::encode_d((double)feq, ref[i]);
-        gd[i * g.npad + s] = Prec<P>::encode_d((double)geq, ref[Q + i]);
-    }
+    equilibria(rho, p, mu, m.Gamma, ux, uy, uz, [&](int i, R feq, R geq) {
+        fd[i * g.npad + s] = Prec<P>::encode_r(feq, ref[i]);
+        gd[i * g.npad + s] = Prec<P>::encode_r(geq, ref[Q + i]);
+    });
 }
 
 // Deviation references from the total of phi (in totals[0]): f_i: w_i rho0;
@@ -373,41 +366,87 @@ __global__ void __launch_bounds__(kRedThreads) k_sum_field(long long n, const do
     block_sum_store<1>(v, partials + (long long)blockIdx.x * kRedFields);
 }
 
+// N consecutive stored values, one load (s a multiple of N).
+template <int N, class S>
+struct alignas(N * sizeof(S)) SiteVec {
+    S v[N];
+};
+// Sites per thread and iteration of k_totals: two where registers allow, to
+// keep more bytes in flight (one site at a time took 0.50 ms at 256^3 in FP32
+// and 1.58 ms in the 16-bit forms, whose 38 references were also read again at
+// every site).
 template <int P>
-__global__ void __launch_bounds__(kRedThreads)
+__host__ __device__ constexpr int totals_sites() {
+    return sizeof(typename Prec<P>::store_t) == 8 ? 1 : 2;
+}
+// Blocks of k_totals: three per SM of the GPU's 152, one wave (a fixed number,
+// so that the order of the sums does not depend on the device).
+constexpr int kTotalsBlocks = 3 * 152;
+
+// Each site's moments are summed in the arithmetic type of the precision (as
+// the step itself forms them); sites accumulate in FP64.
+template <int P>
+__global__ void __launch_bounds__(kRedThreads, 3)
     k_totals(Geom g, const typename Prec<P>::store_t* __restrict__ fs,
-             const typename Prec<P>::store_t* __restrict__ gs, const float* __restrict__ ref,
+             const typename Prec<P>::store_t* __restrict__ gs, const float* __restrict__ ref_g,
              double* __restrict__ partials) {
-    // Each site's moments are summed in the arithmetic type of the precision
-    // (as the step itself forms them); sites accumulate in FP64.
     using R = typename Prec<P>::real_t;
+    using S = typename Prec<P>::store_t;
+    constexpr int N = totals_sites<P>();
+    using V = SiteVec<N, S>;
+    __shared__ float ref[2 * Q];
+    if (threadIdx.x < 2 * Q) ref[threadIdx.x] = ref_g[threadIdx.x];
+    __syncthreads();
+    const volatile float* vref = ref;  // read where used: 38 values held across the loop would spill
     double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < g.n; s += stride) {
-        R rho = R(0), phi = R(0), jx = R(0), jy = R(0), jz = R(0);
+    const long long stride = (long long)gridDim.x * blockDim.x * N;
+    for (long long s = ((long long)blockIdx.x * blockDim.x + threadIdx.x) * N; s < g.n; s += stride) {
+        // npad is a multiple of 64: the last vector may reach past n, into the
+        // row's padding, whose sites are not added
+        V fv[Q], gv[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const R fi = Prec<P>::decode(fs[i * g.npad + s], ref[i]);
-            rho += fi;
-            add_c(i, fi, jx, jy, jz);
-            phi += Prec<P>::decode(gs[i * g.npad + s], ref[Q + i]);
+            fv[i] = *reinterpret_cast<const V*>(fs + i * g.npad + s);
+            gv[i] = *reinterpret_cast<const V*>(gs + i * g.npad + s);
         }
-        v[0] += (double)rho;
-        v[1] += (double)phi;
-        v[2] += (double)jx;
-        v[3] += (double)jy;
-        v[4] += (double)jz;
+        R m[N][5] = {};
+        if constexpr (sizeof(R) == 8) {
+            R f[Q];
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                f[i] = fv[i].v[0];
+                m[0][1] += gv[i].v[0];
+            }
+            moments_f(f, m[0][0], m[0][2], m[0][3], m[0][4]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < Q; ++i) {
+                const float rf = Prec<P>::kDev ? vref[i] : 0.0f, rg = Prec<P>::kDev ? vref[Q + i] : 0.0f;
+#pragma unroll
+                for (int e = 0; e < N; ++e) {
+                    const R fi = Prec<P>::decode(fv[i].v[e], rf);
+                    m[e][0] += fi;
+                    add_c(i, fi, m[e][2], m[e][3], m[e][4]);
+                    m[e][1] += Prec<P>::decode(gv[i].v[e], rg);
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < N; ++e)
+            if (s + e < g.n)
+#pragma unroll
+                for (int k = 0; k < 5; ++k) v[k] += (double)m[e][k];
     }
     block_sum_store<5>(v, partials + (long long)blockIdx.x * kRedFields);
 }
 
-// Final ordered pass: out[k] = sum over blocks of partials[b][k].
-__global__ void __launch_bounds__(kRedBlocks) k_finalize(const double* __restrict__ partials, int nfields,
+// Final ordered pass: out[k] = sum over the nblocks blocks of partials[b][k].
+__global__ void __launch_bounds__(kRedBlocks) k_finalize(const double* __restrict__ partials, int nblocks, int nfields,
                                                          double* __restrict__ out) {
     __shared__ double red[kRedBlocks / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int k = 0; k < nfields; ++k) {
-        double a = partials[(long long)threadIdx.x * kRedFields + k];
+        double a = (int)threadIdx.x < nblocks ? partials[(long long)threadIdx.x * kRedFields + k] : 0.0;
         for (int off = 16; off > 0; off >>= 1) a += __shfl_down_sync(0xffffffffu, a, off);
         if (lane == 0) red[warp] = a;
         __syncthreads();
@@ -422,64 +461,195 @@ __global__ void __launch_bounds__(kRedBlocks) k_finalize(const double* __restric
 
 // ---------------------------------------------------------------------------
 // Macroscopic output (double): rho, u = (j + F/2)/rho, phi, grad phi.
-template <int P>
-__global__ void __launch_bounds__(kThreads)
-    k_macros(Geom g, const typename Prec<P>::store_t* __restrict__ fs,
-             const typename Prec<P>::store_t* __restrict__ gs, const typename Prec<P>::real_t* __restrict__ phis,
-             const typename Prec<P>::real_t* __restrict__ mu, const float* __restrict__ ref,
-             double* __restrict__ rho_out, double* __restrict__ u_out, double* __restrict__ phi_out,
-             double* __restrict__ gphi_out, int iso, const typename Prec<P>::real_t* __restrict__ stress) {
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.n) return;
-    int x, y, z;
-    site_coords(g, s, x, y, z);
-    const int xp = wrap_inc(x, g.nx), xm = wrap_dec(x, g.nx);
-    const int yp = wrap_inc(y, g.ny), ym = wrap_dec(y, g.ny);
-    const int zp = wrap_inc(z, g.nz), zm = wrap_dec(z, g.nz);
-    double rho = 0.0, jx = 0.0, jy = 0.0, jz = 0.0, ph = 0.0;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const double fi = Prec<P>::decode_d(fs[i * g.npad + s], ref[i]);
-        rho += fi;
-        jx += cx(i) * fi;
-        jy += cy(i) * fi;
-        jz += cz(i) * fi;
-        ph += Prec<P>::decode_d(gs[i * g.npad + s], ref[Q + i]);
+//
+// The outputs are FP64, and the FP64 pipe (two instructions per clock and SM)
+// bounds this kernel: with 38 conversions, 95 additions and three divisions a
+// site it took 5.70 ms at 256^3 in FP32 storage, where its bytes need 0.55
+// ms. So FP32 and the 16-bit forms sum the stored values, which are floats, in
+// FP32 arithmetic with every rounding error kept (Sum3), and widen floats to
+// double with integer instructions: 27 FP64 instructions a site. Sites where
+// that is not exact (a sum that leaves the range of floats, values that span
+// more than 48 bits, subnormal values, NaN) take the FP64 form instead, a
+// branch around a call: predicated instructions would occupy the FP64 pipe in
+// every thread (measured: 72 instructions a site, 2.28 ms).
+
+// x as a double times 2^-shift by integer instructions; clears ok unless x
+// is zero or normal.
+template <int shift>
+__device__ __forceinline__ double widen(float x, bool& ok) {
+    const unsigned u = (unsigned)__float_as_int(x), mag = u & 0x7fffffffu;
+    ok = ok && (mag - 0x00800000u < 0x7f000000u || mag == 0u);
+    const unsigned hi = mag == 0u ? 0u : (mag >> 3) + ((896u - shift) << 20);
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+
+// A sum of floats s + e + t with the rounding errors of s kept in e and those
+// of e in t (cascaded summation, Rump, Ogita & Oishi 2008).
+struct Sum3 {
+    float s, e, t;
+    __device__ __forceinline__ static void two_sum(float& a, float b, float& err) {
+        const float r = __fadd_rn(a, b), z = __fsub_rn(r, a);
+        err = __fadd_rn(__fsub_rn(a, __fsub_rn(r, z)), __fsub_rn(b, z));
+        a = r;
     }
-    if (rho_out) rho_out[s] = rho;
-    if (phi_out) phi_out[s] = ph;
-    // gradient of a field (the selected stencil), in FP64
-    auto grad = [&](const typename Prec<P>::real_t* h, double& gx, double& gy, double& gz) {
-        if (iso) {
-            auto nb = [&](int i) {
-                return (double)h[site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny),
-                                         step_coord(z, cz(i), g.nz))];
-            };
-            grad19(nb, gx, gy, gz);
+    __device__ __forceinline__ void add(float x) {
+        float r;
+        two_sum(s, x, r);
+        two_sum(e, r, r);
+        t = __fadd_rn(t, r);
+    }
+    // s + e; clears ok unless that is the whole sum (t is NaN where s overflowed)
+    __device__ __forceinline__ double value(bool& ok) const {
+        ok = ok && t == 0.0f;
+        return widen<0>(s, ok) + widen<0>(e, ok);
+    }
+};
+
+// The arguments of k_macros (outputs may be null).
+template <int P>
+struct MacrosArgs {
+    Geom g;
+    const typename Prec<P>::store_t *fs, *gs;
+    const typename Prec<P>::real_t *phi, *mu, *stress;  // stress: null unless F = -div P
+    const float* ref;
+    double *rho_out, *u_out, *phi_out, *gphi_out;
+    int iso;
+};
+
+// One site. FAST: the float sums and integer conversions above; returns false,
+// with nothing written, where they are not exact. ref_sum: the sums of the
+// references of the deviation forms (sum r_i, sum q_i; r_i = r_-i, so they
+// cancel in j).
+template <int P, bool FAST>
+__device__ __forceinline__ bool macros_site(const MacrosArgs<P>& a, unsigned s, const RowNbr& o, const float* ref,
+                                            const double* ref_sum) {
+    using R = typename Prec<P>::real_t;
+    const long long n = a.g.n, npad = a.g.npad;
+    bool ok = true;
+    double rho, ph, j[3];
+    if constexpr (FAST) {
+        Sum3 r{0.0f, 0.0f, 0.0f}, x = r, y = r, z = r, p = r;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) {
+            const float v = to_float(a.fs[i * npad + s]);
+            r.add(v);
+            if (cx(i) != 0) x.add(cx(i) > 0 ? v : -v);
+            if (cy(i) != 0) y.add(cy(i) > 0 ? v : -v);
+            if (cz(i) != 0) z.add(cz(i) > 0 ? v : -v);
+            p.add(to_float(a.gs[i * npad + s]));
+        }
+        rho = r.value(ok);
+        ph = p.value(ok);
+        j[0] = x.value(ok);
+        j[1] = y.value(ok);
+        j[2] = z.value(ok);
+        if (Prec<P>::kDev) {
+            rho += ref_sum[0];
+            ph += ref_sum[1];
+        }
+    } else {
+        double f[Q];
+#pragma unroll
+        for (int i = 0; i < Q; ++i) f[i] = Prec<P>::decode_d(a.fs[i * npad + s], ref[i]);
+        moments_f(f, rho, j[0], j[1], j[2]);
+        ph = 0.0;
+#pragma unroll
+        for (int i = 0; i < Q; ++i) ph += Prec<P>::decode_d(a.gs[i * npad + s], ref[Q + i]);
+    }
+    // the difference of two field values, and half of it
+    auto diff = [&](const R* h, int d0, int d1) -> double {
+        if constexpr (FAST)
+            return widen<0>(h[s + d0], ok) - widen<0>(h[s + d1], ok);
+        else
+            return (double)h[s + d0] - (double)h[s + d1];
+    };
+    auto half_diff = [&](const R* h, int d0, int d1) -> double {
+        if constexpr (FAST)
+            return widen<1>(h[s + d0], ok) - widen<1>(h[s + d1], ok);
+        else
+            return 0.5 * ((double)h[s + d0] - (double)h[s + d1]);
+    };
+    // gradient of a field with the selected stencil
+    auto grad = [&](const R* h, double (&v)[3]) {
+        if (a.iso) {  // from the differences of opposite neighbours: axis 1/6, diagonal 1/12
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] = 2.0 * diff(h, o.of(2 * c + 1), o.of(2 * c + 2));
+#pragma unroll
+            for (int i = 7; i < Q; i += 2) add_c(i, diff(h, o.of(i), o.of(i + 1)), v[0], v[1], v[2]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] *= 1.0 / 12.0;
         } else {
-            gx = 0.5 * ((double)h[site_of(g, xp, y, z)] - (double)h[site_of(g, xm, y, z)]);
-            gy = 0.5 * ((double)h[site_of(g, x, yp, z)] - (double)h[site_of(g, x, ym, z)]);
-            gz = 0.5 * ((double)h[site_of(g, x, y, zp)] - (double)h[site_of(g, x, y, zm)]);
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[c] = half_diff(h, o.of(2 * c + 1), o.of(2 * c + 2));
         }
     };
-    if (u_out) {
-        double Fx, Fy, Fz;
-        if (stress) {  // F = -div P
+    double u[3], gp[3];
+    if (a.u_out) {
+        double num[3];  // j + F/2
+        if (a.stress) {  // F = -div P
             double d[6][3];
-            for (int c = 0; c < 6; ++c) grad(stress + c * g.npad, d[c][0], d[c][1], d[c][2]);
-            Fx = -((d[0][0] + d[3][1]) + d[4][2]);
-            Fy = -((d[3][0] + d[1][1]) + d[5][2]);
-            Fz = -((d[4][0] + d[5][1]) + d[2][2]);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) grad(a.stress + c * npad, d[c]);
+            num[0] = __fma_rn(-0.5, (d[0][0] + d[3][1]) + d[4][2], j[0]);
+            num[1] = __fma_rn(-0.5, (d[3][0] + d[1][1]) + d[5][2], j[1]);
+            num[2] = __fma_rn(-0.5, (d[4][0] + d[5][1]) + d[2][2], j[2]);
         } else {  // F = -phi grad(mu)
-            double gx, gy, gz;
-            grad(mu, gx, gy, gz);
-            Fx = -ph * gx, Fy = -ph * gy, Fz = -ph * gz;
+            double gm[3];
+            grad(a.mu, gm);
+            const double h = -0.5 * ph;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) num[c] = __fma_rn(h, gm[c], j[c]);
         }
-        u_out[s] = (jx + 0.5 * Fx) / rho;
-        u_out[g.n + s] = (jy + 0.5 * Fy) / rho;
-        u_out[2 * g.n + s] = (jz + 0.5 * Fz) / rho;
+        double inv;
+        if constexpr (FAST) {  // 1/rho to about 46 bits, which the residuals of div_by take to the last
+            const float f = (float)rho;
+            const double r = widen<0>(__frcp_rn(f), ok);
+            ok = ok && fabsf(f) > 1e-30f && fabsf(f) < 1e30f;
+            inv = __fma_rn(__fma_rn(-rho, r, 1.0), r, r);
+        } else {
+            inv = __drcp_rn(rho);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) u[c] = div_by(num[c], rho, inv);
     }
-    if (gphi_out) grad(phis, gphi_out[s], gphi_out[g.n + s], gphi_out[2 * g.n + s]);
+    if (a.gphi_out) grad(a.phi, gp);
+    if (FAST && !ok) return false;
+    if (a.rho_out) a.rho_out[s] = rho;
+    if (a.phi_out) a.phi_out[s] = ph;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        if (a.u_out) a.u_out[c * n + s] = u[c];
+        if (a.gphi_out) a.gphi_out[c * n + s] = gp[c];
+    }
+    return true;
+}
+template <int P>
+__device__ __noinline__ void macros_site_exact(const MacrosArgs<P>& a, unsigned s, const RowNbr& o) {
+    macros_site<P, false>(a, s, o, a.ref, nullptr);
+}
+
+template <int P>
+__global__ void __launch_bounds__(kThreads, 4) k_macros(const __grid_constant__ MacrosArgs<P> a) {
+    constexpr bool kFast = sizeof(typename Prec<P>::store_t) < 8;
+    __shared__ double ref_sum[2];
+    if (Prec<P>::kDev) {
+        if (threadIdx.x < 2) {
+            double v = 0.0;
+            for (int i = 0; i < Q; ++i) v += (double)a.ref[threadIdx.x * Q + i];
+            ref_sum[threadIdx.x] = v;
+        }
+        __syncthreads();
+    }
+    const unsigned s = blockIdx.x * blockDim.x + threadIdx.x;  // n < 2^31
+    if (s >= a.g.n) return;
+    const unsigned row = s / (unsigned)a.g.nx;
+    const int x = (int)(s - row * (unsigned)a.g.nx), z = (int)(row / (unsigned)a.g.ny);
+    const RowNbr o = row_nbr(RowGeom{a.g.nx, a.g.ny, a.g.nz, 0}, x, (int)(row - (unsigned)z * a.g.ny), z);
+    if constexpr (kFast) {
+        if (!macros_site<P, true>(a, s, o, a.ref, ref_sum)) macros_site_exact<P>(a, s, o);
+    } else {
+        macros_site<P, false>(a, s, o, a.ref, nullptr);
+    }
 }
 
 // Distributions out (decoded, stride n) and in (encoded).
@@ -531,7 +701,7 @@ cudaError_t init_p(ld_ctx* c, const double* phi, const double* rho, const double
     if (Prec<P>::kDev) {
         if (!ref_mean) {
             k_sum_field<<<kRedBlocks, kRedThreads, 0, c->stream>>>(g.n, phi, c->partials);
-            k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, 1, c->totals);
+            k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, kRedBlocks, 1, c->totals);
         }
         k_refs<<<1, 32, 0, c->stream>>>(c->totals, g.n, ref_mean ? *ref_mean : 0.0, ref_mean ? 1 : 0, m, c->prm.rho0,
                                         c->ref);
@@ -614,10 +784,9 @@ cudaError_t macros_p(ld_ctx* c, double* rho, double* u, double* phi, double* gph
             k_stress<R, long long><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
                 row_geom(c->geom), (long long)g.npad, model_of<R>(c->prm), (const R*)c->phi, (R*)c->stress);
     }
-    k_macros<P><<<blocks_for(g.n), kThreads, 0, c->stream>>>(g, (const S*)f_of(c, c->cur), (const S*)g_of(c, c->cur),
-                                                             (const R*)c->phi, (const R*)c->mu, c->ref, rho, u,
-                                                             phi, gphi, c->prm.stencil == LD_STENCIL_19,
-                                                             (const R*)c->stress);
+    k_macros<P><<<blocks_for(g.n), kThreads, 0, c->stream>>>(
+        MacrosArgs<P>{g, (const S*)f_of(c, c->cur), (const S*)g_of(c, c->cur), (const R*)c->phi, (const R*)c->mu,
+                      (const R*)c->stress, c->ref, rho, u, phi, gphi, c->prm.stencil == LD_STENCIL_19});
     return cudaGetLastError();
 }
 
@@ -625,9 +794,9 @@ template <int P>
 cudaError_t totals_p(ld_ctx* c, double* out) {
     using S = typename Prec<P>::store_t;
     const Geom g = to_dev(c->geom);
-    k_totals<P><<<kRedBlocks, kRedThreads, 0, c->stream>>>(g, (const S*)f_of(c, c->cur), (const S*)g_of(c, c->cur),
+    k_totals<P><<<kTotalsBlocks, kRedThreads, 0, c->stream>>>(g, (const S*)f_of(c, c->cur), (const S*)g_of(c, c->cur),
                                                            c->ref, c->partials);
-    k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, 5, out);
+    k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, kTotalsBlocks, 5, out);
     return cudaGetLastError();
 }
 

@@ -68,7 +68,7 @@ bool staged_supported(int nx, int ny, int nz, int prec) {
 cudaError_t launch_propagate(ld_ctx* c, int reverse) { return propagate_raw(c, reverse); }
 cudaError_t launch_field_sum(ld_ctx* c, long long n, const double* x, double* out) {
     k_sum_field<<<kRedBlocks, kRedThreads, 0, c->stream>>>(n, x, c->partials);
-    k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, 1, out);
+    k_finalize<<<1, kRedBlocks, 0, c->stream>>>(c->partials, kRedBlocks, 1, out);
     return cudaGetLastError();
 }
 cudaError_t launch_default_refs(ld_ctx* c) { return default_refs(c); }

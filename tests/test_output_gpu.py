@@ -1,0 +1,116 @@
+"""Initial state and macroscopic output on the GPU where their FP32-pipe forms
+could go wrong: rounding of the 16-bit initial deviations, the moments' error-
+free float sums and integer conversions at extreme values, lattices whose
+size is not a multiple of the vectors that the totals load."""
+
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_1609_01479_gb300 import inputs, ld  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+STORE = {"fp32": torch.float32, "fp16dev": torch.float16, "bf16dev": torch.bfloat16, "fp64": torch.float64}
+
+
+def planes(sim, precision):
+    nz, ny, nx = sim.shape
+    out = torch.empty((38, nz, ny, nx), dtype=STORE[precision], device="cuda")
+    ld.ld_pack_planes(sim.ctx, 0, nz, out)
+    return out
+
+
+def round_once(x, bits, emin):
+    """float64 x rounded to nearest even with `bits` significant bits and least exponent emin."""
+    _, e = np.frexp(x)
+    step = np.ldexp(1.0, np.maximum(e - bits, emin - bits + 1))
+    return np.rint(x / step) * step
+
+
+@pytest.mark.parametrize("precision,bits,emin", [("fp16dev", 11, -14), ("bf16dev", 8, -126)])
+def test_initial_deviations_are_rounded_once(precision, bits, emin):
+    """At rest f_i = w_i rho, one FP32 product. With rho away from rho0 = 1 the FP32 difference to the
+    reference is inexact, and rounding it again would differ from rounding the exact one."""
+    nx, ny, nz = 40, 12, 9
+    phi = np.zeros((nz, ny, nx))
+    rho = np.random.default_rng(4).uniform(0.1, 8.0, phi.shape)
+    sim = ld.LdSim(nx, ny, nz, precision=precision)
+    sim.init(torch.from_numpy(phi).cuda(), torch.from_numpy(rho).cuda())
+    got = planes(sim, precision)[:19].double().cpu().numpy()
+    w = np.array([np.float32(1) / np.float32(3)] + [np.float32(1) / np.float32(18)] * 6
+                 + [np.float32(1) / np.float32(36)] * 12, np.float32)[:, None, None, None]
+    ref = np.array([1 / 3] + [1 / 18] * 6 + [1 / 36] * 12).astype(np.float32)[:, None, None, None]
+    exact = (w * rho.astype(np.float32)).astype(np.float64) - ref.astype(np.float64)
+    once = round_once(exact, bits, emin)
+    assert np.array_equal(got, once)
+    twice = round_once(exact.astype(np.float32).astype(np.float64), bits, emin)
+    assert precision == "bf16dev" or (twice != once).any()
+
+
+@pytest.mark.parametrize("case", ["ordinary", "wide", "subnormal", "huge", "inf", "nan", "zero"])
+@pytest.mark.parametrize("stencil", [7, 19])
+def test_moments_of_extreme_states(case, stencil):
+    nx, ny, nz = 11, 6, 5
+    rng = np.random.default_rng(5)
+    f = rng.random((19, nz, ny, nx)) * 0.1 + 0.01
+    g = rng.standard_normal((19, nz, ny, nx)) * 0.1
+    if case == "wide":  # values spanning more bits than a double holds
+        g *= np.float64(2.0) ** rng.integers(-70, 5, g.shape)
+    elif case == "subnormal":
+        g *= 2.0 ** -130
+    elif case == "huge":  # the float sum overflows, the double one does not
+        f[:, 1, 2, 3] = 3.0e38
+    elif case == "inf":
+        f[4, 1, 2, 3] = math.inf
+        g[7, 2, 1, 0] = -math.inf
+    elif case == "nan":
+        f[4, 1, 2, 3] = math.nan
+    elif case == "zero":
+        g[:] = 0.0
+    f, g = (a.astype(np.float32).astype(np.float64) for a in (f, g))  # what the state holds
+    sim = ld.LdSim(nx, ny, nz, precision="fp32", stencil=stencil)
+    sim.set_distributions(torch.from_numpy(f), torch.from_numpy(g))
+    m = {k: v.cpu().numpy() for k, v in sim.moments(grad_phi=True).items()}
+    exact = lambda a: np.array([math.fsum(v) if np.isfinite(v).all() else v.sum()  # noqa: E731
+                                for v in a.reshape(19, -1).T]).reshape(a.shape[1:])
+    # a sum of 19 doubles is within 18 units of 2^-53 of the sum of magnitudes
+    for key, a in (("rho", f), ("phi", g)):
+        want, tol = exact(a), 18 * 2.0 ** -53 * np.abs(a).sum(axis=0)
+        fine = np.isfinite(want)
+        assert np.array_equal(np.isnan(m[key]), np.isnan(want))
+        assert np.array_equal(m[key][~fine & ~np.isnan(want)], want[~fine & ~np.isnan(want)])
+        assert (np.abs(m[key] - want)[fine] <= tol[fine]).all()
+    if case in ("ordinary", "wide", "zero"):  # u = (j + F/2)/rho with F = -phi grad(mu) of the FP32 mu
+        assert np.isfinite(m["u"]).all() and np.isfinite(m["grad_phi"]).all()
+        phi32 = np.zeros(g.shape[1:], np.float32)
+        for i in range(19):
+            phi32 = phi32 + g[i].astype(np.float32)
+        roll = lambda h, a, d: np.roll(h, -d, axis=2 - a)  # noqa: E731
+        p = phi32.astype(np.float64)
+        if stencil == 7:
+            want = np.stack([0.5 * (roll(p, a, 1) - roll(p, a, -1)) for a in range(3)])
+            assert np.abs(m["grad_phi"] - want).max() <= 2.0 ** -53 * np.abs(p).max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16dev", "bf16dev"])
+@pytest.mark.parametrize("dims", [(5, 5, 5), (33, 7, 5), (64, 8, 4), (31, 30, 29)])
+def test_totals_of_sizes_off_the_vectors(precision, dims):
+    nx, ny, nz = dims
+    sim = ld.LdSim(nx, ny, nz, precision=precision)
+    sim.workspace.fill_(255)  # NaN in the padding of every row, which must not be added
+    sim.close()
+    sim.ctx = ld.ld_create(nx, ny, nz, sim.params, sim.workspace)
+    sim.init(torch.from_numpy(inputs.spinodal_phi(nx, ny, nz, seed=6, amplitude=0.4)).cuda())
+    f, g = (t.cpu().numpy() for t in sim.distributions())
+    got = sim.totals().cpu().numpy()
+    n = nx * ny * nz
+    # each site's 19 values are summed in the arithmetic type: at most 18 roundings of the sum of magnitudes
+    unit = 2.0 ** -53 if precision == "fp64" else 2.0 ** -24
+    want = np.array([f.sum(), g.sum()])
+    tol = 20 * unit * np.array([np.abs(f).sum(), np.abs(g).sum()]) + n * 2.0 ** -52
+    assert (np.abs(got[:2] - want) <= tol).all()
+    assert np.abs(got[2:]).max() <= 20 * unit * np.abs(f).sum()
