@@ -66,8 +66,9 @@ enum { LD_FP64 = 0, LD_FP32 = 1, LD_FP16DEV = 2, LD_BF16DEV = 3 };
  *   (cp.async, completion tracked on mbarriers with bounded waits); FP32 and
  *   the 16-bit forms only (nx % 32 == 0, ny % 8 == 0, nz % 4 == 0); every
  *   stencil and rounding option of FUSED.
- * LD_KERNEL_AUTO: FUSED when the lattice admits it, else GENERIC; always
- * GENERIC for LD_FP64, which is bound by the FP64 pipe, where the generic
+ * LD_KERNEL_AUTO: FUSED when the lattice admits it, else GENERIC (in
+ *   LD_FP32 a small lattice of any size runs a one-launch kernel of its own,
+ *   with the same results); always GENERIC for LD_FP64, which is bound by the FP64 pipe, where the generic
  * launches do less FP64 work per site (no halo phi sums). */
 enum { LD_KERNEL_AUTO = 0, LD_KERNEL_GENERIC = 1, LD_KERNEL_FUSED = 2, LD_KERNEL_FUSED_STAGED = 3 };
 
@@ -213,7 +214,9 @@ int ld_unpack_planes(ld_ctx* ctx, int z0, int nplanes, const void* dev_buf);
 
 /* The step kernel a context runs (LD_KERNEL_AUTO resolved for its lattice,
  * precision and options): LD_KERNEL_GENERIC, LD_KERNEL_FUSED or
- * LD_KERNEL_FUSED_STAGED; LD_EINVAL for a NULL context. */
+ * LD_KERNEL_FUSED_STAGED; LD_EINVAL for a NULL context. Where AUTO runs its
+ * small-lattice kernel: the one it would resolve to for a larger lattice of
+ * the same divisibility. */
 int ld_step_kernel(const ld_ctx* ctx);
 
 /* Advance nsteps >= 0 full timesteps (moments, phi stencil and mu, force,

@@ -358,6 +358,11 @@ int ld_step_kernel(const ld_ctx* c) {
         case ld::kStepGeneric: return LD_KERNEL_GENERIC;
         case ld::kStepRegs: return LD_KERNEL_FUSED;
         case ld::kStepStaged: return LD_KERNEL_FUSED_STAGED;
+        // AUTO on a small lattice, whose one launch does the step of either
+        case ld::kStepSmall:
+            return ld::choose_step_kernel(c->geom.nx, c->geom.ny, c->geom.nz, c->prec, LD_KERNEL_FUSED)
+                       ? LD_KERNEL_FUSED
+                       : LD_KERNEL_GENERIC;
         default: return LD_EINVAL;
     }
 }

@@ -113,6 +113,7 @@ inline void* g_of(const ld_ctx* c, int buf) { return g_part(c, c->dist[buf]); }
     cudaError_t encode(ld_ctx* c, const double* f, const double* g);                              \
     cudaError_t step_fused_regs(ld_ctx* c, const void* src, void* dst, void* fields);             \
     cudaError_t step_staged(ld_ctx* c, const void* src, void* dst, void* fields);                 \
+    cudaError_t step_small(ld_ctx* c, const void* src, void* dst, void* fields);                  \
     cudaError_t adj_step(ld_ctx* c, const void* state_t, const void* fields_t, double* grad);     \
     cudaError_t adj_seed(ld_ctx* c, const double* phibar);                                        \
     cudaError_t adj_init(ld_ctx* c, const double* phi0, const double* u0, double* gphi0, double* grad); \
@@ -148,7 +149,7 @@ cudaError_t set_max_dynamic_smem_once(int bytes) {
 }
 
 // Step kernels (ld_ctx::step_kernel).
-enum StepKernel { kStepGeneric = 1, kStepStaged = 2, kStepRegs = 3 };
+enum StepKernel { kStepGeneric = 1, kStepStaged = 2, kStepRegs = 3, kStepSmall = 4 };
 // The kernel a request resolves to for this lattice and precision, or 0 if
 // the requested one cannot run it.
 int choose_step_kernel(int nx, int ny, int nz, int prec, int requested);
@@ -195,6 +196,7 @@ inline cudaError_t launch_step(ld_ctx* c, const void* src, void* dst, void* fiel
         return is_f64(c) ? f64::collide_generic(c, src, dst, fields) : lp::collide_generic(c, src, dst, fields);
     if (c->step_kernel == kStepStaged)
         return is_f64(c) ? f64::step_staged(c, src, dst, fields) : lp::step_staged(c, src, dst, fields);
+    if (c->step_kernel == kStepSmall) return lp::step_small(c, src, dst, fields);
     return is_f64(c) ? f64::step_fused_regs(c, src, dst, fields) : lp::step_fused_regs(c, src, dst, fields);
 }
 

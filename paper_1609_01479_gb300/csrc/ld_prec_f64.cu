@@ -27,6 +27,8 @@ cudaError_t step_fused_regs(ld_ctx* c, const void* src, void* dst, void* fields)
 }
 // FP64 staging would not fit shared memory at the occupancy the FP64 pipe needs
 cudaError_t step_staged(ld_ctx*, const void*, void*, void*) { return cudaErrorNotSupported; }
+// the FP64 pipe bounds small lattices too, and the halo's phi sums would add to it
+cudaError_t step_small(ld_ctx*, const void*, void*, void*) { return cudaErrorNotSupported; }
 bool regs_supported(int nx, int ny, int nz) { return fused_supported_impl(nx, ny, nz); }
 cudaError_t adj_step(ld_ctx* c, const void* st, const void* fields, double* grad) {
     return adj_step_p<LD_FP64>(c, st, fields, grad);

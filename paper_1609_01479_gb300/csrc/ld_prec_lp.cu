@@ -3,6 +3,7 @@
 #include "ld_fused.cuh"
 #include "ld_fused2.cuh"
 #include "ld_generic.cuh"
+#include "ld_small.cuh"
 #include "ld_staged.cuh"
 #include "ld_adjoint.cuh"
 
@@ -40,6 +41,9 @@ cudaError_t step_fused_regs(ld_ctx* c, const void* src, void* dst, void* fields)
 }
 cudaError_t step_staged(ld_ctx* c, const void* src, void* dst, void* fields) {
     LD_LP_DISPATCH(step_staged_p, c, src, dst, fields);
+}
+cudaError_t step_small(ld_ctx* c, const void* src, void* dst, void* fields) {
+    return launch_small(c, src, dst, fields);
 }
 bool regs_supported(int nx, int ny, int nz) { return fused_supported_impl(nx, ny, nz); }
 cudaError_t adj_step(ld_ctx* c, const void* st, const void* fields, double* grad) {
@@ -82,7 +86,9 @@ int choose_step_kernel(int nx, int ny, int nz, int prec, int requested) {
         case LD_KERNEL_FUSED_STAGED: return staged ? kStepStaged : 0;
         // FP64 is bound by the FP64 pipe, and the three row-ordered launches
         // do less FP64 work per site than the fused step (no halo phi sums)
-        case LD_KERNEL_AUTO: return regs && !f64p ? kStepRegs : kStepGeneric;
+        case LD_KERNEL_AUTO:
+            if (prec == LD_FP32 && small_supported_impl(nx, ny, nz)) return kStepSmall;
+            return regs && !f64p ? kStepRegs : kStepGeneric;
         default: return 0;
     }
 }
