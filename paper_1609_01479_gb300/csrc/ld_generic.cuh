@@ -19,10 +19,10 @@ inline Geom to_dev(const GeomH& h) { return Geom{h.nx, h.ny, h.nz, h.n, h.npad};
 inline unsigned blocks_for(long long n) { return (unsigned)((n + kThreads - 1) / kThreads); }
 
 __device__ __forceinline__ void site_coords(const Geom& g, long long s, int& x, int& y, int& z) {
-    x = (int)(s % g.nx);
-    long long t = s / g.nx;
-    y = (int)(t % g.ny);
-    z = (int)(t / g.ny);
+    const unsigned i = (unsigned)s, t = i / (unsigned)g.nx;  // n < 2^31 (ld_create)
+    x = (int)(i - t * (unsigned)g.nx);
+    z = (int)(t / (unsigned)g.ny);
+    y = (int)(t - (unsigned)z * (unsigned)g.ny);
 }
 
 __device__ __forceinline__ long long site_of(const Geom& g, int x, int y, int z) {
@@ -35,45 +35,79 @@ __device__ __forceinline__ int step_coord(int a, int d, int n) {
 }
 
 // ---------------------------------------------------------------------------
-// The step as three launches in site order, one thread per site, each block
-// a segment of kRowThreads sites of one x-row (a block never straddles two
-// rows, so the coordinates need one division per thread).
-// Consecutive blocks cover consecutive addresses of every stream, the order
-// that lets HBM run at its copy rate. Element offsets i npad + s are of type
-// I: 32-bit where 19 npad fits.
+// The step as launches in site order, kRowThreads consecutive sites per block,
+// across the ends of rows: consecutive blocks cover consecutive addresses of
+// every stream, the order that lets HBM run at its copy rate, and every block
+// is full whatever nx is (blocks of one row's sites left 41 % of the threads
+// idle at nx = 150). A site's coordinates come from its index by two
+// multiplications (FastDiv). Element offsets i npad + s are of type I: 32-bit
+// where 19 npad fits.
+
+// Quotient of 0 <= a < 2^31 by a fixed 2 <= d < 2^31 (Granlund & Montgomery
+// 1994): m = ceil(2^(31+l)/d) < 2^32 with l = ceil(log2 d), q = a m / 2^(31+l).
+struct FastDiv {
+    unsigned m;
+    int shift;
+    __device__ __forceinline__ int div(int a) const { return (int)(__umulhi((unsigned)a, m) >> shift); }
+};
+inline FastDiv fast_div(int d) {
+    int l = 1;
+    while ((1LL << l) < d) ++l;
+    return FastDiv{(unsigned)(((1ULL << (31 + l)) + (unsigned)d - 1) / (unsigned)d), l - 1};
+}
+
 struct RowGeom {
-    int nx, ny, nz, nchunks;  // nchunks = blocks per row
+    int nx, ny, nz, n;
+    FastDiv dx, dy;
 };
 
 inline RowGeom row_geom(const GeomH& h) {
-    return RowGeom{h.nx, h.ny, h.nz, (h.nx + kRowThreads - 1) / kRowThreads};
+    return RowGeom{h.nx, h.ny, h.nz, (int)h.n, fast_div(h.nx), fast_div(h.ny)};
 }
 
-inline unsigned row_blocks(const GeomH& h) { return (unsigned)row_segments(h); }
+inline unsigned row_blocks(const GeomH& h) { return (unsigned)((h.n + kRowThreads - 1) / kRowThreads); }
 
-// Site of this thread in row segment b (false past the end of its row).
-__device__ __forceinline__ bool row_site(const RowGeom& rg, int b, int& x, int& y, int& z, int& s) {
-    const int r = b / rg.nchunks;
-    x = (b - r * rg.nchunks) * kRowThreads + threadIdx.x;
-    y = r % rg.ny;
-    z = r / rg.ny;
-    s = r * rg.nx + x;
-    return x < rg.nx;
+// Site of this thread (false past the end of the lattice).
+__device__ __forceinline__ bool row_site(const RowGeom& rg, int& x, int& y, int& z, int& s) {
+    s = (int)(blockIdx.x * kRowThreads + threadIdx.x);
+    if ((unsigned)s >= (unsigned)rg.n) return false;
+    const int row = rg.dx.div(s);
+    x = s - row * rg.nx;
+    z = rg.dy.div(row);
+    y = row - z * rg.ny;
+    return true;
 }
 
-// Stage 1: phi = sum_i g_i (the stored state is the post-propagation one).
-template <int P, class I>
-__global__ void __launch_bounds__(kRowThreads) k_phi(RowGeom rg, I npad, const typename Prec<P>::store_t* __restrict__ gs,
+// N consecutive stored values, one load (s a multiple of N).
+template <int N, class S>
+struct alignas(N * sizeof(S)) SiteVec {
+    S v[N];
+};
+
+// Stage 1: phi = sum_i g_i (the stored state is the post-propagation one), two
+// sites per thread with 32- and 16-bit storage. npad is even: the second site
+// may be the first of the padding, whose phi nothing reads.
+template <int P>
+__host__ __device__ constexpr int phi_sites() {
+    return sizeof(typename Prec<P>::store_t) == 8 ? 1 : 2;
+}
+template <int P, class I, int N>
+__global__ void __launch_bounds__(kRowThreads) k_phi(int n, I npad, const typename Prec<P>::store_t* __restrict__ gs,
                                                      const float* __restrict__ ref,
                                                      typename Prec<P>::real_t* __restrict__ phi, int* __restrict__ status) {
     using R = typename Prec<P>::real_t;
-    int x, y, z, s;
-    if (!row_site(rg, blockIdx.x, x, y, z, s)) return;
-    if (!site_ok(s, (long long)rg.nx * rg.ny * rg.nz, status)) return;
-    R acc = R(0);
+    using S = typename Prec<P>::store_t;
+    const int s = (int)((blockIdx.x * kRowThreads + threadIdx.x) * N);
+    if ((unsigned)s >= (unsigned)n || !site_ok(s, n, status)) return;
+    SiteVec<N, S> v[Q];
 #pragma unroll
-    for (int i = 0; i < Q; ++i) acc += Prec<P>::decode(gs[i * npad + s], ref[Q + i]);
-    phi[s] = acc;
+    for (int i = 0; i < Q; ++i) v[i] = *reinterpret_cast<const SiteVec<N, S>*>(gs + i * npad + s);
+    SiteVec<N, R> acc{};
+#pragma unroll
+    for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int e = 0; e < N; ++e) acc.v[e] += Prec<P>::decode(v[i].v[e], ref[Q + i]);
+    *reinterpret_cast<SiteVec<N, R>*>(phi + s) = acc;
 }
 
 // Stage 2: mu = A phi + B phi^3 - kappa lap(phi), with the 7-point or the
@@ -82,7 +116,7 @@ template <class R>
 __global__ void __launch_bounds__(kRowThreads) k_mu(RowGeom rg, Model<R> m, const R* __restrict__ phi,
                                                     R* __restrict__ mu) {
     int x, y, z, s;
-    if (!row_site(rg, blockIdx.x, x, y, z, s)) return;
+    if (!row_site(rg, x, y, z, s)) return;
     const int nx = rg.nx, plane = rg.nx * rg.ny;
     const int xp = x + 1 == nx ? 1 - nx : 1, xm = x == 0 ? nx - 1 : -1;
     const int yp = y + 1 == rg.ny ? (1 - rg.ny) * nx : nx, ym = y == 0 ? (rg.ny - 1) * nx : -nx;
@@ -135,12 +169,13 @@ __device__ __forceinline__ void grad_at(int iso, const T* h, int s, const RowNbr
 // xz, yz) from grad phi and lap(phi) with the selected stencils:
 //   iso = A/2 phi^2 + 3B/4 phi^4 - kappa phi lap - kappa/2 |grad phi|^2,
 //   P_aa = iso + kappa (d_a phi)^2, P_ab = kappa d_a phi d_b phi,
-// each expression in that operation order.
+// each expression in that operation order. Takes the place of k_mu: the step
+// needs mu at the site alone with this force, and it has the Laplacian at hand.
 template <class R, class I>
 __global__ void __launch_bounds__(kRowThreads) k_stress(RowGeom rg, I npad, Model<R> m, const R* __restrict__ phi,
-                                                        R* __restrict__ P) {
+                                                        R* __restrict__ P, R* __restrict__ mu) {
     int x, y, z, s;
-    if (!row_site(rg, blockIdx.x, x, y, z, s)) return;
+    if (!row_site(rg, x, y, z, s)) return;
     const RowNbr o = row_nbr(rg, x, y, z);
     const R ph = phi[s];
     R gx, gy, gz, lap;
@@ -148,8 +183,11 @@ __global__ void __launch_bounds__(kRowThreads) k_stress(RowGeom rg, I npad, Mode
     if (m.iso) {
         auto nb = [&](int i) { return phi[s + o.of(i)]; };
         lap = lap19(ph, nb);
+        mu[s] = chem_potential_lap(ph, lap, m);
     } else {
-        lap = phi[s + o.xp] + phi[s + o.xm] + phi[s + o.yp] + phi[s + o.ym] + phi[s + o.zp] + phi[s + o.zm] - R(6) * ph;
+        const R nb = phi[s + o.xp] + phi[s + o.xm] + phi[s + o.yp] + phi[s + o.ym] + phi[s + o.zp] + phi[s + o.zm];
+        mu[s] = chem_potential(ph, nb, m);
+        lap = nb - R(6) * ph;
     }
     const R pb = R(0.5) * m.A * ph * ph + R(0.75) * m.B * ph * ph * ph * ph;
     const R iso = pb - m.kappa * ph * lap - R(0.5) * m.kappa * (gx * gx + gy * gy + gz * gz);
@@ -174,31 +212,66 @@ __device__ __forceinline__ void stress_force_at(int iso, const T* P, I npad, int
     Fz = -((d[4][0] + d[5][1]) + d[2][2]);
 }
 
-// Resident blocks per SM the collision kernel is compiled for: 6 x 128
-// threads (80 registers) with FP32 arithmetic, 3 with FP64.
+// grad mu by central differences (as unscaled differences, twice the gradient)
+// and mu at a site from phi alone: mu at the site and its six neighbours, each
+// the operations of k_mu, from the 25 phi within two sites.
+template <class R>
+__device__ __forceinline__ void mu_diffs_of_phi(const RowGeom& rg, const Model<R>& m, const R* phi, int x, int y, int z,
+                                                int s, const RowNbr& o, R& mu, R& dx, R& dy, R& dz) {
+    const int nx = rg.nx, plane = rg.nx * rg.ny;
+    const int x2 = x + 2 >= nx ? 2 - nx : 2, xm2 = x < 2 ? nx - 2 : -2;
+    const int y2 = (y + 2 >= rg.ny ? 2 - rg.ny : 2) * nx, ym2 = (y < 2 ? rg.ny - 2 : -2) * nx;
+    const int z2 = (z + 2 >= rg.nz ? 2 - rg.nz : 2) * plane, zm2 = (z < 2 ? rg.nz - 2 : -2) * plane;
+    const R* p = phi + s;
+    const R c = p[0], xp = p[o.xp], xm = p[o.xm], yp = p[o.yp], ym = p[o.ym], zp = p[o.zp], zm = p[o.zm];
+    const R xpyp = p[o.xp + o.yp], xpym = p[o.xp + o.ym], xmyp = p[o.xm + o.yp], xmym = p[o.xm + o.ym];
+    const R xpzp = p[o.xp + o.zp], xpzm = p[o.xp + o.zm], xmzp = p[o.xm + o.zp], xmzm = p[o.xm + o.zm];
+    const R ypzp = p[o.yp + o.zp], ypzm = p[o.yp + o.zm], ymzp = p[o.ym + o.zp], ymzm = p[o.ym + o.zm];
+    mu = chem_potential(c, xp + xm + yp + ym + zp + zm, m);
+    dx = chem_potential(xp, p[x2] + c + xpyp + xpym + xpzp + xpzm, m) -
+         chem_potential(xm, c + p[xm2] + xmyp + xmym + xmzp + xmzm, m);
+    dy = chem_potential(yp, xpyp + xmyp + p[y2] + c + ypzp + ypzm, m) -
+         chem_potential(ym, xpym + xmym + c + p[ym2] + ymzp + ymzm, m);
+    dz = chem_potential(zp, xpzp + xmzp + ypzp + ymzp + p[z2] + c, m) -
+         chem_potential(zm, xpzm + xmzm + ypzm + ymzm + c + p[zm2], m);
+}
+
+// Whether the step's collision forms mu from phi itself (mu_diffs_of_phi) and
+// k_mu is not launched: with the 7-point stencils and the potential force,
+// except in FP64, where seven mu per site would add 60 FP64 instructions.
 template <int P>
+bool near_mu(const ld_ctx* c) {
+    return sizeof(typename Prec<P>::real_t) == 4 && !c->stress && c->prm.stencil == LD_STENCIL_7;
+}
+
+// Resident blocks per SM the collision kernel is compiled for: 6 x 128
+// threads (80 registers) with FP32 arithmetic, 5 (96) where it forms mu from
+// phi, 3 with FP64.
+template <int P, bool NEAR>
 constexpr int rows_blocks_per_sm() {
-    return sizeof(typename Prec<P>::real_t) == 4 ? 6 : 3;
+    return sizeof(typename Prec<P>::real_t) == 4 ? (NEAR ? 5 : 6) : 3;
 }
 
 // Stage 3: force, velocity, collisions of f and g, and propagation (push: the
 // post-collision value of direction i goes to x + c_i) with streaming stores;
-// SR: the 16-bit stores rounded stochastically from the stream `sr`.
-template <int P, class I, bool SR>
-__global__ void __launch_bounds__(kRowThreads, rows_blocks_per_sm<P>())
+// NEAR: mu and its gradient formed here from phi (mu_out, when not null,
+// receives mu); SR: the 16-bit stores rounded stochastically from `sr`.
+template <int P, class I, bool NEAR, bool SR>
+__global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
     k_collide(RowGeom rg, I npad, Model<typename Prec<P>::real_t> m, SrStream sr, const typename Prec<P>::store_t* __restrict__ fs,
               const typename Prec<P>::store_t* __restrict__ gs, typename Prec<P>::store_t* __restrict__ fd,
               typename Prec<P>::store_t* __restrict__ gd, const typename Prec<P>::real_t* __restrict__ phi,
               const typename Prec<P>::real_t* __restrict__ mu, const float* __restrict__ ref,
-              const typename Prec<P>::real_t* __restrict__ stress, int* __restrict__ status) {
+              const typename Prec<P>::real_t* __restrict__ stress, typename Prec<P>::real_t* __restrict__ mu_out,
+              int* __restrict__ status) {
     using R = typename Prec<P>::real_t;
     using S = typename Prec<P>::store_t;
     __shared__ float refs[2 * Q];  // codec references, read once per block
     if (threadIdx.x < 2 * Q) refs[threadIdx.x] = ref[threadIdx.x];
     __syncthreads();
     int x, y, z, s;
-    if (!row_site(rg, blockIdx.x, x, y, z, s)) return;
-    const long long n = (long long)rg.nx * rg.ny * rg.nz;
+    if (!row_site(rg, x, y, z, s)) return;
+    const long long n = rg.n;
     if (!site_ok(s, n, status)) return;
     // FP32 and FP64 issue all 38 loads first; the 16-bit forms issue g after
     // the f stores (each 16-bit value held early would take a register).
@@ -209,18 +282,20 @@ __global__ void __launch_bounds__(kRowThreads, rows_blocks_per_sm<P>())
         fr[i] = __ldcs(fs + i * npad + s);
         if (kEarlyG) gr[i] = __ldcs(gs + i * npad + s);
     }
-    const int nx = rg.nx, plane = rg.nx * rg.ny;
-    const int oxp = x + 1 == nx ? 1 - nx : 1, oxm = x == 0 ? nx - 1 : -1;
-    const int oyp = y + 1 == rg.ny ? (1 - rg.ny) * nx : nx, oym = y == 0 ? (rg.ny - 1) * nx : -nx;
-    const int ozp = z + 1 == rg.nz ? (1 - rg.nz) * plane : plane, ozm = z == 0 ? (rg.nz - 1) * plane : -plane;
-
-    const R ph = phi[s], muc = mu[s];
-    const RowNbr o{oxp, oxm, oyp, oym, ozp, ozm};
-    R Fx, Fy, Fz;
-    if (stress) {  // F = -div P
-        stress_force_at(m.iso, stress, npad, s, o, Fx, Fy, Fz);
-    } else {  // F = -phi grad(mu)
-        if (m.iso) {
+    const RowNbr o = row_nbr(rg, x, y, z);
+    const int oxp = o.xp, oxm = o.xm, oyp = o.yp, oym = o.ym, ozp = o.zp, ozm = o.zm;
+    const R ph = phi[s];
+    R muc, Fx, Fy, Fz;
+    if constexpr (NEAR) {
+        R dx, dy, dz;
+        mu_diffs_of_phi(rg, m, phi, x, y, z, s, o, muc, dx, dy, dz);
+        force_of_diffs(ph, dx, dy, dz, Fx, Fy, Fz);
+        if (mu_out) mu_out[s] = muc;
+    } else {
+        muc = mu[s];
+        if (stress) {  // F = -div P
+            stress_force_at(m.iso, stress, npad, s, o, Fx, Fy, Fz);
+        } else if (m.iso) {  // F = -phi grad(mu)
             R gmx, gmy, gmz;
             grad_at(1, mu, s, o, gmx, gmy, gmz);
             Fx = -ph * gmx, Fy = -ph * gmy, Fz = -ph * gmz;
@@ -366,11 +441,6 @@ __global__ void __launch_bounds__(kRedThreads) k_sum_field(long long n, const do
     block_sum_store<1>(v, partials + (long long)blockIdx.x * kRedFields);
 }
 
-// N consecutive stored values, one load (s a multiple of N).
-template <int N, class S>
-struct alignas(N * sizeof(S)) SiteVec {
-    S v[N];
-};
 // Sites per thread and iteration of k_totals: two where registers allow, to
 // keep more bytes in flight (one site at a time took 0.50 ms at 256^3 in FP32
 // and 1.58 ms in the 16-bit forms, whose 38 references were also read again at
@@ -525,18 +595,20 @@ __device__ __forceinline__ bool macros_site(const MacrosArgs<P>& a, unsigned s, 
                                             const double* ref_sum) {
     using R = typename Prec<P>::real_t;
     const long long n = a.g.n, npad = a.g.npad;
+    const bool need_f = a.rho_out || a.u_out;
     bool ok = true;
-    double rho, ph, j[3];
+    double rho = 0.0, ph, j[3];
     if constexpr (FAST) {
         Sum3 r{0.0f, 0.0f, 0.0f}, x = r, y = r, z = r, p = r;
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
+            p.add(to_float(a.gs[i * npad + s]));
+            if (!need_f) continue;
             const float v = to_float(a.fs[i * npad + s]);
             r.add(v);
             if (cx(i) != 0) x.add(cx(i) > 0 ? v : -v);
             if (cy(i) != 0) y.add(cy(i) > 0 ? v : -v);
             if (cz(i) != 0) z.add(cz(i) > 0 ? v : -v);
-            p.add(to_float(a.gs[i * npad + s]));
         }
         rho = r.value(ok);
         ph = p.value(ok);
@@ -548,10 +620,12 @@ __device__ __forceinline__ bool macros_site(const MacrosArgs<P>& a, unsigned s, 
             ph += ref_sum[1];
         }
     } else {
-        double f[Q];
+        if (need_f) {
+            double f[Q];
 #pragma unroll
-        for (int i = 0; i < Q; ++i) f[i] = Prec<P>::decode_d(a.fs[i * npad + s], ref[i]);
-        moments_f(f, rho, j[0], j[1], j[2]);
+            for (int i = 0; i < Q; ++i) f[i] = Prec<P>::decode_d(a.fs[i * npad + s], ref[i]);
+            moments_f(f, rho, j[0], j[1], j[2]);
+        }
         ph = 0.0;
 #pragma unroll
         for (int i = 0; i < Q; ++i) ph += Prec<P>::decode_d(a.gs[i * npad + s], ref[Q + i]);
@@ -644,7 +718,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_macros(const __grid_constant__ 
     if (s >= a.g.n) return;
     const unsigned row = s / (unsigned)a.g.nx;
     const int x = (int)(s - row * (unsigned)a.g.nx), z = (int)(row / (unsigned)a.g.ny);
-    const RowNbr o = row_nbr(RowGeom{a.g.nx, a.g.ny, a.g.nz, 0}, x, (int)(row - (unsigned)z * a.g.ny), z);
+    const RowNbr o = row_nbr(RowGeom{a.g.nx, a.g.ny, a.g.nz, 0, {}, {}}, x, (int)(row - (unsigned)z * a.g.ny), z);
     if constexpr (kFast) {
         if (!macros_site<P, true>(a, s, o, a.ref, ref_sum)) macros_site_exact<P>(a, s, o);
     } else {
@@ -714,59 +788,84 @@ cudaError_t init_p(ld_ctx* c, const double* phi, const double* rho, const double
     return cudaGetLastError();
 }
 
-// phi and mu of a state into `fields` ([phi npad][mu npad]), or into the
-// context's scratch when fields is null.
+inline bool offsets_fit_int(const ld_ctx* c) { return (long long)Q * c->geom.npad <= 0x7fffffffLL; }
+
 template <int P, class I>
-cudaError_t phi_mu_rows(ld_ctx* c, const void* state, void* fields) {
+void launch_phi(ld_ctx* c, const void* state, typename Prec<P>::real_t* phi) {
     using S = typename Prec<P>::store_t;
-    using R = typename Prec<P>::real_t;
-    const RowGeom rg = row_geom(c->geom);
+    constexpr int N = phi_sites<P>();
+    const S* gs = (const S*)g_part(c, state);
     const unsigned nb = row_blocks(c->geom);
-    R* phi = fields ? (R*)fields : (R*)c->phi;
-    R* mu = fields ? (R*)fields + c->geom.npad : (R*)c->mu;
-    k_phi<P, I><<<nb, kRowThreads, 0, c->stream>>>(rg, (I)c->geom.npad, (const S*)g_part(c, state), c->ref, phi,
-                                                   c->status);
-    k_mu<R><<<nb, kRowThreads, 0, c->stream>>>(rg, model_of<R>(c->prm), phi, mu);
+    // a caller's state or fields buffer may be aligned to single values only
+    if (N > 1 && (uintptr_t)gs % (N * sizeof(S)) == 0 && (uintptr_t)phi % (N * sizeof(*phi)) == 0)
+        k_phi<P, I, N><<<(nb + N - 1) / N, kRowThreads, 0, c->stream>>>((int)c->geom.n, (I)c->geom.npad, gs, c->ref, phi,
+                                                                        c->status);
+    else
+        k_phi<P, I, 1><<<nb, kRowThreads, 0, c->stream>>>((int)c->geom.n, (I)c->geom.npad, gs, c->ref, phi, c->status);
+}
+
+// mu from phi, and the chemical stress where the force is its divergence.
+template <class R, class I>
+void launch_mu(ld_ctx* c, const R* phi, R* mu) {
+    const unsigned nb = row_blocks(c->geom);
+    if (c->stress)
+        k_stress<R, I><<<nb, kRowThreads, 0, c->stream>>>(row_geom(c->geom), (I)c->geom.npad, model_of<R>(c->prm), phi,
+                                                          (R*)c->stress, mu);
+    else
+        k_mu<R><<<nb, kRowThreads, 0, c->stream>>>(row_geom(c->geom), model_of<R>(c->prm), phi, mu);
+}
+
+// phi and mu of a state (and the stress) into the context's scratch.
+template <int P>
+cudaError_t phi_mu_p(ld_ctx* c, const void* state) {
+    using R = typename Prec<P>::real_t;
+    if (offsets_fit_int(c)) {
+        launch_phi<P, int>(c, state, (R*)c->phi);
+        launch_mu<R, int>(c, (const R*)c->phi, (R*)c->mu);
+    } else {
+        launch_phi<P, long long>(c, state, (R*)c->phi);
+        launch_mu<R, long long>(c, (const R*)c->phi, (R*)c->mu);
+    }
     return cudaGetLastError();
 }
 
-inline bool offsets_fit_int(const ld_ctx* c) { return (long long)Q * c->geom.npad <= 0x7fffffffLL; }
-
-template <int P>
-cudaError_t phi_mu_p(ld_ctx* c, const void* state, void* fields = nullptr) {
-    return offsets_fit_int(c) ? phi_mu_rows<P, int>(c, state, fields) : phi_mu_rows<P, long long>(c, state, fields);
-}
-
-template <int P, class I, bool SR>
+// One step; phi and mu of the source state go to `fields` ([phi npad][mu
+// npad]) when it is not null, else to the context's scratch.
+template <int P, class I, bool NEAR, bool SR>
 cudaError_t collide_rows(ld_ctx* c, const void* src, void* dst, void* fields) {
     using S = typename Prec<P>::store_t;
     using R = typename Prec<P>::real_t;
-    cudaError_t e = phi_mu_rows<P, I>(c, src, fields);
-    if (e != cudaSuccess) return e;
-    const R* phi = fields ? (const R*)fields : (const R*)c->phi;
-    const R* mu = fields ? (const R*)fields + c->geom.npad : (const R*)c->mu;
-    if (c->stress)
-        k_stress<R, I><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(row_geom(c->geom), (I)c->geom.npad,
-                                                                           model_of<R>(c->prm), phi, (R*)c->stress);
-    k_collide<P, I, SR><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
+    R* phi = fields ? (R*)fields : (R*)c->phi;
+    R* mu = fields ? (R*)fields + c->geom.npad : (R*)c->mu;
+    launch_phi<P, I>(c, src, phi);
+    if (!NEAR) launch_mu<R, I>(c, phi, mu);
+    k_collide<P, I, NEAR, SR><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
         row_geom(c->geom), (I)c->geom.npad, model_of<R>(c->prm), sr_stream(c->prm.seed, c->sr_step, c->geom.n),
-        (const S*)f_part(c, src), (const S*)g_part(c, src),
-        (S*)f_part(c, dst), (S*)g_part(c, dst), phi, mu, c->ref, (const R*)c->stress, c->status);
+        (const S*)f_part(c, src), (const S*)g_part(c, src), (S*)f_part(c, dst), (S*)g_part(c, dst), phi,
+        NEAR ? nullptr : mu, c->ref, (const R*)c->stress, NEAR && fields ? mu : nullptr, c->status);
     return cudaGetLastError();
 }
 
-template <int P, bool SR>
+template <int P, bool NEAR, bool SR>
 cudaError_t collide_r(ld_ctx* c, const void* src, void* dst, void* fields) {
-    return offsets_fit_int(c) ? collide_rows<P, int, SR>(c, src, dst, fields)
-                              : collide_rows<P, long long, SR>(c, src, dst, fields);
+    return offsets_fit_int(c) ? collide_rows<P, int, NEAR, SR>(c, src, dst, fields)
+                              : collide_rows<P, long long, NEAR, SR>(c, src, dst, fields);
+}
+
+template <int P, bool SR>
+cudaError_t collide_n(ld_ctx* c, const void* src, void* dst, void* fields) {
+    if constexpr (sizeof(typename Prec<P>::real_t) == 4) {
+        if (near_mu<P>(c)) return collide_r<P, true, SR>(c, src, dst, fields);
+    }
+    return collide_r<P, false, SR>(c, src, dst, fields);
 }
 
 template <int P>
 cudaError_t collide_p(ld_ctx* c, const void* src, void* dst, void* fields) {
     if constexpr (Prec<P>::kDev) {
-        if (c->prm.rounding == LD_ROUND_STOCHASTIC) return collide_r<P, true>(c, src, dst, fields);
+        if (c->prm.rounding == LD_ROUND_STOCHASTIC) return collide_n<P, true>(c, src, dst, fields);
     }
-    return collide_r<P, false>(c, src, dst, fields);
+    return collide_n<P, false>(c, src, dst, fields);
 }
 
 template <int P>
@@ -774,15 +873,9 @@ cudaError_t macros_p(ld_ctx* c, double* rho, double* u, double* phi, double* gph
     using S = typename Prec<P>::store_t;
     using R = typename Prec<P>::real_t;
     const Geom g = to_dev(c->geom);
-    cudaError_t e = phi_mu_p<P>(c, c->dist[c->cur]);
-    if (e != cudaSuccess) return e;
-    if (c->stress) {
-        if (offsets_fit_int(c))
-            k_stress<R, int><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
-                row_geom(c->geom), (int)g.npad, model_of<R>(c->prm), (const R*)c->phi, (R*)c->stress);
-        else
-            k_stress<R, long long><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
-                row_geom(c->geom), (long long)g.npad, model_of<R>(c->prm), (const R*)c->phi, (R*)c->stress);
+    if (u || gphi) {
+        const cudaError_t e = phi_mu_p<P>(c, c->dist[c->cur]);
+        if (e != cudaSuccess) return e;
     }
     k_macros<P><<<blocks_for(g.n), kThreads, 0, c->stream>>>(
         MacrosArgs<P>{g, (const S*)f_of(c, c->cur), (const S*)g_of(c, c->cur), (const R*)c->phi, (const R*)c->mu,
