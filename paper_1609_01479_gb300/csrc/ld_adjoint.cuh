@@ -35,18 +35,25 @@ namespace {
 
 constexpr int kAdjThreads = 256;
 
-// Fixed-order block sum of one double per thread into out[0] (thread 0 writes).
+// Fixed-order block sum of one double per thread into out[0]: the first warp
+// adds the others' values, eight per lane, then its lanes. The FP64 pipe takes
+// 12 instructions a block for it; a shuffle tree in every warp took 40, which
+// made the sums of k_adj_mu cost more than its memory traffic.
 __device__ __forceinline__ void block_sum_one(double v, double* out) {
-    __shared__ double red[kAdjThreads / 32];
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) red[warp] = v;
+    __shared__ double red[kAdjThreads];
+    red[threadIdx.x] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0;
-        for (int w = 0; w < kAdjThreads / 32; ++w) a += red[w];
-        *out = a;
-    }
+    if (threadIdx.x >= 32) return;
+#pragma unroll
+    for (int w = 1; w < kAdjThreads / 32; ++w) v += red[threadIdx.x + 32 * w];
+    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+    if (threadIdx.x == 0) *out = v;
+}
+
+// Site s of a lattice (s < n < 2^31) and its neighbours' offsets.
+__device__ __forceinline__ RowNbr site_nbr(const RowGeom& rg, int s) {
+    const int row = rg.dx.div(s), z = rg.dy.div(row);
+    return row_nbr(rg, s - row * rg.nx, row - z * rg.ny, z);
 }
 
 // Two resident 256-thread CTAs per SM for the local adjoint kernel: at three
@@ -57,9 +64,9 @@ constexpr int adj_ctas_per_sm() {
 }
 
 // Step 1 + 2: local adjoint at every site.
-template <int P, bool ISO>
+template <int P, class I, bool ISO>
 __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<P>())
-    k_adj_local(Geom g, Model<typename Prec<P>::real_t> m, const typename Prec<P>::store_t* __restrict__ tf,
+    k_adj_local(RowGeom rg, I npad, Model<typename Prec<P>::real_t> m, const typename Prec<P>::store_t* __restrict__ tf,
                 const typename Prec<P>::real_t* __restrict__ phi, const typename Prec<P>::real_t* __restrict__ mu,
                 const float* __restrict__ ref, const typename Prec<P>::real_t* __restrict__ fb1,
                 const typename Prec<P>::real_t* __restrict__ gb1, const typename Prec<P>::real_t* __restrict__ pb1,
@@ -67,28 +74,15 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<P>())
                 typename Prec<P>::real_t* __restrict__ gmb, typename Prec<P>::real_t* __restrict__ mub,
                 typename Prec<P>::real_t* __restrict__ phib, double* __restrict__ part) {
     using R = typename Prec<P>::real_t;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int s = (int)(blockIdx.x * kAdjThreads + threadIdx.x);
     double omega_bar = 0.0;
-    if (s < g.n) {
-        typename Prec<P>::real_t omega_site = 0;
-        int x, y, z;
-        site_coords(g, s, x, y, z);
-        const int xp = wrap_inc(x, g.nx), xm = wrap_dec(x, g.nx);
-        const int yp = wrap_inc(y, g.ny), ym = wrap_dec(y, g.ny);
-        const int zp = wrap_inc(z, g.nz), zm = wrap_dec(z, g.nz);
+    if ((unsigned)s < (unsigned)rg.n) {
+        R omega_site = 0;
+        const RowNbr o = site_nbr(rg, s);
         // forward quantities
         const R ph = phi[s];
         R gmx, gmy, gmz;
-        if constexpr (ISO) {
-            auto nb = [&](int i) {
-                return mu[site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny), step_coord(z, cz(i), g.nz))];
-            };
-            grad19(nb, gmx, gmy, gmz);
-        } else {
-            gmx = R(0.5) * (mu[site_of(g, xp, y, z)] - mu[site_of(g, xm, y, z)]);
-            gmy = R(0.5) * (mu[site_of(g, x, yp, z)] - mu[site_of(g, x, ym, z)]);
-            gmz = R(0.5) * (mu[site_of(g, x, y, zp)] - mu[site_of(g, x, y, zm)]);
-        }
+        grad_at(ISO, mu, s, o, gmx, gmy, gmz);
         const R Fx = -ph * gmx, Fy = -ph * gmy, Fz = -ph * gmz;
         // reverse propagation: the values pushed from x along c_i. They do
         // not depend on the forward moments, so they are loaded together with
@@ -96,16 +90,15 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<P>())
         R fbs[Q], gbs[Q];
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const long long o = site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny),
-                                        step_coord(z, cz(i), g.nz));
-            fbs[i] = fb1[i * g.npad + o];
-            gbs[i] = gb1[i * g.npad + o] + pb1[o];
+            const int d = s + o.of(i);
+            fbs[i] = fb1[i * npad + d];
+            gbs[i] = gb1[i * npad + d] + pb1[d];
         }
         R f[Q];
         R rho = R(0), jx = R(0), jy = R(0), jz = R(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            f[i] = Prec<P>::decode(tf[i * g.npad + s], ref[i]);
+            f[i] = Prec<P>::decode(tf[i * npad + s], ref[i]);
             rho += f[i];
             add_c(i, f[i], jx, jy, jz);
         }
@@ -123,7 +116,7 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<P>())
         R phib_l = R(0), mub_l = R(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            gb0[i * g.npad + s] = (R(1) - m.omega_g) * gbs[i];
+            gb0[i * npad + s] = (R(1) - m.omega_g) * gbs[i];
             const R w = wgt<R>(i);
             const R cu = cdot(i, ux, uy, uz);
             const R cF = cdot(i, Fx, Fy, Fz);
@@ -161,101 +154,123 @@ __global__ void __launch_bounds__(kAdjThreads, adj_ctas_per_sm<P>())
         // F = -phi gm
         phib_l -= Fbx * gmx + Fby * gmy + Fbz * gmz;
         gmb[s] = -ph * Fbx;
-        gmb[g.npad + s] = -ph * Fby;
-        gmb[2 * g.npad + s] = -ph * Fbz;
+        gmb[npad + s] = -ph * Fby;
+        gmb[2 * npad + s] = -ph * Fbz;
         mub[s] = mub_l;
         phib[s] = phib_l;
         omega_bar = (double)omega_site;
         // fbar at t: direct term + rho and j
 #pragma unroll
         for (int i = 0; i < Q; ++i)
-            fb0[i * g.npad + s] = (R(1) - m.omega_f) * fbs[i] + rhob + cdot(i, jbx, jby, jbz);
+            fb0[i * npad + s] = (R(1) - m.omega_f) * fbs[i] + rhob + cdot(i, jbx, jby, jbz);
     }
     block_sum_one(omega_bar, part + 2 * (long long)blockIdx.x);
 }
 
+// FP64 sum of products of floats (or doubles) of one thread. Float products
+// and their sum are formed in FP32 with every rounding error kept (Sum3, and
+// the error of a product by one fused operation), so that the FP64 pipe takes
+// five instructions a thread instead of four a product; products that FP32
+// does not hold exactly that way (overflow, underflow, NaN) are added in FP64.
+template <class R>
+struct ProductSum;
+template <>
+struct ProductSum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { v += a * b; }
+    __device__ __forceinline__ double value() const { return v; }
+};
+template <>
+struct ProductSum<float> {
+    Sum3 a{0.0f, 0.0f, 0.0f};
+    double rest = 0.0;
+    __device__ __forceinline__ void add(float x, float y) {
+        const float p = __fmul_rn(x, y), m = fabsf(p);
+        if (m >= 1e-30f && m <= 1e30f) {
+            a.add(p);
+            a.add(__fmaf_rn(x, y, -p));
+        } else if (p != 0.0f || x != 0.0f) {
+            rest += (double)x * (double)y;
+        }
+    }
+    __device__ __forceinline__ double value() const { return rest + ((double)a.s + ((double)a.e + (double)a.t)); }
+};
+
+// Sites per thread of k_adj_mu, kAdjThreads apart.
+constexpr int kAdjMuSites = 4;
+
 // Step 3: mubar += transpose of the gradient applied to gmbar; kappa
 // partials mubar (-lap phi). 7-point: the transposed central difference;
 // 19-point: mubar(y) += sum_i 3 w_i c_i . gmbar(y - c_i).
-template <class R, bool ISO>
+template <class R, class I, bool ISO>
 __global__ void __launch_bounds__(kAdjThreads)
-    k_adj_mu(Geom g, const R* __restrict__ phi, const R* __restrict__ gmb, R* __restrict__ mub,
+    k_adj_mu(RowGeom rg, I npad, const R* __restrict__ phi, const R* __restrict__ gmb, R* __restrict__ mub,
              double* __restrict__ part) {
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    double kappa_bar = 0.0;
-    if (s < g.n) {
-        int x, y, z;
-        site_coords(g, s, x, y, z);
+    ProductSum<R> kappa_bar;
+#pragma unroll
+    for (int k = 0; k < kAdjMuSites; ++k) {
+        const int s = (int)((blockIdx.x * kAdjMuSites + k) * kAdjThreads + threadIdx.x);
+        if ((unsigned)s >= (unsigned)rg.n) break;
+        const RowNbr o = site_nbr(rg, s);
+        const R *gx = gmb + s, *gy = gmb + npad + s, *gz = gmb + 2 * npad + s;
         R t, lap;
         if constexpr (ISO) {
             t = mub[s];
             lap = R(0);
 #pragma unroll
             for (int i = 1; i < Q; ++i) {
-                const long long back = site_of(g, step_coord(x, -cx(i), g.nx), step_coord(y, -cy(i), g.ny),
-                                               step_coord(z, -cz(i), g.nz));
-                const long long fwd = site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny),
-                                              step_coord(z, cz(i), g.nz));
-                const R dot = cdot(i, gmb[back], gmb[g.npad + back], gmb[2 * g.npad + back]);
-                t += grad19_coef<R>(i) * dot;
-                lap += lap19_coef<R>(i) * (phi[fwd] - phi[s]);
+                const int back = o.of(i & 1 ? i + 1 : i - 1);  // the opposite direction
+                t += grad19_coef<R>(i) * cdot(i, gx[back], gy[back], gz[back]);
+                lap += lap19_coef<R>(i) * (phi[s + o.of(i)] - phi[s]);
             }
         } else {
-            const long long sxm = site_of(g, wrap_dec(x, g.nx), y, z), sxp = site_of(g, wrap_inc(x, g.nx), y, z);
-            const long long sym = site_of(g, x, wrap_dec(y, g.ny), z), syp = site_of(g, x, wrap_inc(y, g.ny), z);
-            const long long szm = site_of(g, x, y, wrap_dec(z, g.nz)), szp = site_of(g, x, y, wrap_inc(z, g.nz));
-            t = mub[s] + R(0.5) * (gmb[sxm] - gmb[sxp]) + R(0.5) * (gmb[g.npad + sym] - gmb[g.npad + syp]) +
-                R(0.5) * (gmb[2 * g.npad + szm] - gmb[2 * g.npad + szp]);
-            lap = phi[sxp] + phi[sxm] + phi[syp] + phi[sym] + phi[szp] + phi[szm] - R(6) * phi[s];
+            t = mub[s] + R(0.5) * (gx[o.xm] - gx[o.xp]) + R(0.5) * (gy[o.ym] - gy[o.yp]) +
+                R(0.5) * (gz[o.zm] - gz[o.zp]);
+            lap = phi[s + o.xp] + phi[s + o.xm] + phi[s + o.yp] + phi[s + o.ym] + phi[s + o.zp] + phi[s + o.zm] -
+                  R(6) * phi[s];
         }
         mub[s] = t;
-        kappa_bar = -(double)t * (double)lap;
+        kappa_bar.add(-t, lap);
     }
-    block_sum_one(kappa_bar, part + 2 * (long long)blockIdx.x + 1);
+    block_sum_one(kappa_bar.value(), part + 2 * (long long)blockIdx.x + 1);
 }
 
 // Laplacian (7-point or 19-point, symmetric: its own transpose) of a field
-// at site s = (x, y, z), in the type of the field.
+// at site s, in the type of the field.
 template <bool ISO, class T>
-__device__ __forceinline__ T lap_at(const Geom& g, const T* h, long long s, int x, int y, int z) {
+__device__ __forceinline__ T lap_at(const T* h, int s, const RowNbr& o) {
     if constexpr (ISO) {
         T lap = T(0);
 #pragma unroll
-        for (int i = 1; i < Q; ++i)
-            lap += lap19_coef<T>(i) *
-                   (h[site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny), step_coord(z, cz(i), g.nz))] -
-                    h[s]);
+        for (int i = 1; i < Q; ++i) lap += lap19_coef<T>(i) * (h[s + o.of(i)] - h[s]);
         return lap;
     }
-    return h[site_of(g, wrap_inc(x, g.nx), y, z)] + h[site_of(g, wrap_dec(x, g.nx), y, z)] +
-           h[site_of(g, x, wrap_inc(y, g.ny), z)] + h[site_of(g, x, wrap_dec(y, g.ny), z)] +
-           h[site_of(g, x, y, wrap_inc(z, g.nz))] + h[site_of(g, x, y, wrap_dec(z, g.nz))] - T(6) * h[s];
+    return h[s + o.xp] + h[s + o.xm] + h[s + o.yp] + h[s + o.ym] + h[s + o.zp] + h[s + o.zm] - T(6) * h[s];
 }
 
 // Step 4: phibar, the per-site part P of gbar at t.
 template <class R, bool ISO>
 __global__ void __launch_bounds__(kAdjThreads)
-    k_adj_p(Geom g, Model<R> m, const R* __restrict__ phi, const R* __restrict__ mub, const R* __restrict__ phib,
+    k_adj_p(RowGeom rg, Model<R> m, const R* __restrict__ phi, const R* __restrict__ mub, const R* __restrict__ phib,
             R* __restrict__ pb0) {
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= g.n) return;
-    int x, y, z;
-    site_coords(g, s, x, y, z);
+    const int s = (int)(blockIdx.x * kAdjThreads + threadIdx.x);
+    if ((unsigned)s >= (unsigned)rg.n) return;
     const R ph = phi[s];
-    const R lapm = lap_at<ISO>(g, mub, s, x, y, z);
+    const R lapm = lap_at<ISO>(mub, s, site_nbr(rg, s));
     pb0[s] = phib[s] + (m.A + R(3) * m.B * ph * ph) * mub[s] - m.kappa * lapm;
 }
 
-// grad[0] += sum_b part[2b+1] (kappa); grad[1] += taub_scale * sum_b part[2b]
-// (tau_f); one block, fixed order.
-__global__ void __launch_bounds__(kAdjThreads)
-    k_adj_finalize(const double* __restrict__ part, long long nblk, double taub_scale, double* __restrict__ grad) {
-    __shared__ double red[2][kAdjThreads / 32];
+// grad[0] += the sum of part[2b + 1] over b < nkappa (kappa); grad[1] +=
+// taub_scale * the sum of part[2b] over b < ntau (tau_f); one block, fixed
+// order.
+constexpr int kAdjFinalThreads = 1024;
+__global__ void __launch_bounds__(kAdjFinalThreads)
+    k_adj_finalize(const double* __restrict__ part, int nkappa, int ntau, double taub_scale, double* __restrict__ grad) {
+    __shared__ double red[2][kAdjFinalThreads / 32];
     double a = 0.0, b = 0.0;
-    for (long long k = threadIdx.x; k < nblk; k += kAdjThreads) {
-        a += part[2 * k + 1];
-        b += part[2 * k];
-    }
+    for (long long k = threadIdx.x; k < nkappa; k += kAdjFinalThreads) a += part[2 * k + 1];
+#pragma unroll 4
+    for (long long k = threadIdx.x; k < ntau; k += kAdjFinalThreads) b += part[2 * k];
     for (int off = 16; off > 0; off >>= 1) {
         a += __shfl_down_sync(0xffffffffu, a, off);
         b += __shfl_down_sync(0xffffffffu, b, off);
@@ -268,7 +283,7 @@ __global__ void __launch_bounds__(kAdjThreads)
     __syncthreads();
     if (threadIdx.x == 0) {
         double ka = 0.0, tb = 0.0;
-        for (int w = 0; w < kAdjThreads / 32; ++w) {
+        for (int w = 0; w < kAdjFinalThreads / 32; ++w) {
             ka += red[0][w];
             tb += red[1][w];
         }
@@ -311,14 +326,13 @@ __global__ void __launch_bounds__(kAdjThreads)
 // Per-site sums in the arithmetic type; outputs and partials in FP64.
 template <class R, bool ISO>
 __global__ void __launch_bounds__(kAdjThreads)
-    k_adj_init_phi(Geom g, Model<R> m, const double* __restrict__ phi0, const double* __restrict__ u0,
+    k_adj_init_phi(Geom g, RowGeom rg, Model<R> m, const double* __restrict__ phi0, const double* __restrict__ u0,
                    const R* __restrict__ gb, const R* __restrict__ pb, const R* __restrict__ mub,
                    double* __restrict__ grad_phi0, double* __restrict__ part) {
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     double kappa_bar = 0.0;
     if (s < g.n) {
-        int x, y, z;
-        site_coords(g, s, x, y, z);
+        const RowNbr o = site_nbr(rg, (int)s);
         R ux = R(0), uy = R(0), uz = R(0);
         if (u0) {
             ux = (R)u0[s];
@@ -336,9 +350,9 @@ __global__ void __launch_bounds__(kAdjThreads)
         }
         const R ph = (R)phi0[s];
         const R mb = mub[s];
-        const R lapm = lap_at<ISO>(g, mub, s, x, y, z);
+        const R lapm = lap_at<ISO>(mub, (int)s, o);
         grad_phi0[s] = (double)(acc + (m.A + R(3) * m.B * ph * ph) * mb - m.kappa * lapm);
-        const double lap = lap_at<ISO>(g, phi0, s, x, y, z);
+        const double lap = lap_at<ISO>(phi0, (int)s, o);
         kappa_bar = -(double)mb * lap;
     }
     if (threadIdx.x == 0) part[2 * (long long)blockIdx.x] = 0.0;  // no tau_f term in the initialiser
@@ -389,34 +403,42 @@ AdjPtrs<P> adj_ptrs(ld_ctx* c, int in_buf) {
     return p;
 }
 
-template <int P, bool ISO>
+template <int P, class I, bool ISO>
 cudaError_t adj_step_iso(ld_ctx* c, const void* state_t, const void* fields_t, double* grad) {
     using S = typename Prec<P>::store_t;
     using R = typename Prec<P>::real_t;
-    const Geom g = to_dev(c->geom);
+    const RowGeom rg = row_geom(c->geom);
+    const I npad = (I)c->geom.npad;
     if (!fields_t) {
         cudaError_t e = phi_mu_p<P>(c, state_t);
         if (e != cudaSuccess) return e;
     }
     const R* phi = fields_t ? (const R*)fields_t : (const R*)c->phi;
-    const R* mu = fields_t ? (const R*)fields_t + g.npad : (const R*)c->mu;
+    const R* mu = fields_t ? (const R*)fields_t + c->geom.npad : (const R*)c->mu;
     const AdjPtrs<P> p = adj_ptrs<P>(c, c->adj_cur);
     const Model<R> m = model_of<R>(c->prm);
-    const unsigned nb = blocks_for(g.n);
-    k_adj_local<P, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, m, (const S*)f_part(c, state_t), phi, mu, c->ref, p.fb1,
-                                                      p.gb1, p.pb1, p.fb0, p.gb0, p.gmb, p.mub, p.phib, c->adj_part);
-    k_adj_mu<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, phi, p.gmb, p.mub, c->adj_part);
-    k_adj_p<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, m, phi, p.mub, p.phib, p.pb0);
+    const unsigned nb = blocks_for(c->geom.n), nbm = (nb + kAdjMuSites - 1) / kAdjMuSites;
+    k_adj_local<P, I, ISO><<<nb, kAdjThreads, 0, c->stream>>>(rg, npad, m, (const S*)f_part(c, state_t), phi, mu, c->ref,
+                                                              p.fb1, p.gb1, p.pb1, p.fb0, p.gb0, p.gmb, p.mub, p.phib,
+                                                              c->adj_part);
+    k_adj_mu<R, I, ISO><<<nbm, kAdjThreads, 0, c->stream>>>(rg, npad, phi, p.gmb, p.mub, c->adj_part);
+    k_adj_p<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(rg, m, phi, p.mub, p.phib, p.pb0);
     if (grad)
-        k_adj_finalize<<<1, kAdjThreads, 0, c->stream>>>(c->adj_part, nb, -1.0 / (c->prm.tau_f * c->prm.tau_f),
-                                                         grad);
+        k_adj_finalize<<<1, kAdjFinalThreads, 0, c->stream>>>(c->adj_part, (int)nbm, (int)nb,
+                                                              -1.0 / (c->prm.tau_f * c->prm.tau_f), grad);
     return cudaGetLastError();
+}
+
+template <int P, bool ISO>
+cudaError_t adj_step_off(ld_ctx* c, const void* state_t, const void* fields_t, double* grad) {
+    return offsets_fit_int(c) ? adj_step_iso<P, int, ISO>(c, state_t, fields_t, grad)
+                              : adj_step_iso<P, long long, ISO>(c, state_t, fields_t, grad);
 }
 
 template <int P>
 cudaError_t adj_step_p(ld_ctx* c, const void* state_t, const void* fields_t, double* grad) {
-    return c->prm.stencil == LD_STENCIL_19 ? adj_step_iso<P, true>(c, state_t, fields_t, grad)
-                                           : adj_step_iso<P, false>(c, state_t, fields_t, grad);
+    return c->prm.stencil == LD_STENCIL_19 ? adj_step_off<P, true>(c, state_t, fields_t, grad)
+                                           : adj_step_off<P, false>(c, state_t, fields_t, grad);
 }
 
 template <int P>
@@ -435,9 +457,9 @@ cudaError_t adj_init_iso(ld_ctx* c, const double* phi0, const double* u0, double
     const AdjPtrs<P> p = adj_ptrs<P>(c, c->adj_cur);
     const unsigned nb = blocks_for(g.n);
     k_adj_init_mu<R><<<nb, kAdjThreads, 0, c->stream>>>(g, (R)c->prm.Gamma, p.gb1, p.pb1, p.mub);
-    k_adj_init_phi<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, model_of<R>(c->prm), phi0, u0, p.gb1, p.pb1, p.mub,
+    k_adj_init_phi<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, row_geom(c->geom), model_of<R>(c->prm), phi0, u0, p.gb1, p.pb1, p.mub,
                                                          grad_phi0, c->adj_part);
-    if (grad) k_adj_finalize<<<1, kAdjThreads, 0, c->stream>>>(c->adj_part, nb, 0.0, grad);
+    if (grad) k_adj_finalize<<<1, kAdjFinalThreads, 0, c->stream>>>(c->adj_part, (int)nb, (int)nb, 0.0, grad);
     return cudaGetLastError();
 }
 
