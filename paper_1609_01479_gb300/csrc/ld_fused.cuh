@@ -24,6 +24,8 @@
 // Template only: instantiated per storage precision by ld_prec_f64.cu and
 // ld_prec_lp.cu.
 #pragma once
+#include <math.h>
+
 #include "ld_common.cuh"
 #include "ld_internal.h"
 #include "ld_async.cuh"
@@ -336,30 +338,30 @@ __global__ void __launch_bounds__(kTX * TY, fused_ctas_per_sm<P>())
 constexpr int kTY = 8;
 
 // z-chunks per tile column. Each CTA marches one chunk of the nz planes,
-// chunk b spanning [chunk_begin(b), chunk_begin(b + 1)). The chunk length zc
-// is the divisor of nz among 64, 32, ..., 4 that minimises
-//   (zc + 4) x (columns x m / (per_sm x SMs) + 0.6),   m = nz / zc:
-// each CTA pays a prologue of about four planes (four extra phi planes, two
-// mu planes and the pipeline start), the m chunks of every column are spread
-// over the resident CTA slots, and the tail of the launch costs about 0.6 of
-// one chunk (CTAs are scheduled as slots free up, so less than a whole
-// wave). The weights reproduce the measured order of the lengths (fraction of
-// measured HBM): 256^3 FP32 32 (0.728) > 16 (0.718) > 8 (0.706) > 64 (0.666);
-// 256^3 16-bit pairs 16 (0.545) ~ 32 (0.542) > 64 (0.519) ~ 8 (0.514); 384^3
-// FP32 64 ahead of 32 and 16 (16.4 k against 15.5-15.8 k MLUPS). Chunks of
-// any length (nz split into m near-equal parts) measured no faster for FP32
-// and 10 % slower for the 16-bit pairs at 384^3.
+// chunk b spanning [chunk_begin(b), chunk_begin(b + 1)), lengths that differ by
+// at most one plane. The number of chunks m (4 planes or more each) minimises
+//   (longest chunk + 1) x (w + 0.9 / (1 + (c - 1)/2) x (c - w)),
+// w = columns x m / resident CTA slots the waves of CTAs and c = ceil(w): a
+// chunk costs its planes and a prologue worth about one more (its loads
+// overlap the other CTAs' work), and the empty slots of the last wave cost the
+// less the more waves there are to drift apart. So m fills whole waves where
+// few make up the launch: a launch of 2.25 waves of 8-plane chunks ran 147 us
+// where one wave of 18 planes takes 130 (128^3 FP32; powers of two only,
+// before). Fitted to 48 measured sweeps over m (three precisions, 64^3 to
+// 384^3 and flat or tall lattices); us a step with the powers of two and now:
+// FP32 128^3 147 and 130, 64 x 64 x 128 64 and 39, 160^3 277 and 255, 224^3 765
+// and 715, 256^3 1037 and 1020, 384^3 3447 and 3440; FP16-dev 128^3 107 and 99,
+// 160^3 188 and 169, 224^3 491 and 445, 256^3 695 and 657; BF16-dev 256^3 649
+// and 625, 352 x 72 x 36 54 and 47.
 int choose_chunks(int nx, int ny, int nz, int rows, int num_sms = 152, int per_sm = 2) {
-    const long long cols = (long long)(nx / kTX) * (ny / rows);
-    const long long slots = (long long)per_sm * num_sms;
-    int best = 0;
-    long long best_cost = 0;
-    for (int zc = 64; zc >= 4; zc /= 2) {
-        if (nz % zc) continue;
-        const long long m = nz / zc;
-        const long long cost = (zc + 4) * (10 * cols * m + 6 * slots);  // x 10 slots
-        if (best == 0 || cost < best_cost) {
-            best = (int)m;
+    const double cols = (double)(nx / kTX) * (ny / rows), slots = (double)per_sm * num_sms;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int m = 1; m <= nz / 4; ++m) {
+        const double w = cols * m / slots, c = ceil(w);
+        const double cost = ((nz + m - 1) / m + 1) * (w + 0.9 / (0.5 + 0.5 * c) * (c - w));
+        if (m == 1 || cost < best_cost) {
+            best = m;
             best_cost = cost;
         }
     }
