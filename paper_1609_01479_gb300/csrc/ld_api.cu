@@ -118,6 +118,17 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Whether both pointers are device memory of one GPU (the copy kernel cannot
+// reach another GPU's memory, the runtime's copies can).
+bool on_one_device(const void* p, const void* q) {
+    cudaPointerAttributes a, b;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, q) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && b.type == cudaMemoryTypeDevice && a.device == b.device;
+}
+
 bool opt_device(const void* p) { return p == nullptr || is_device_ptr(p); }
 
 int check_ready(ld_ctx* c) {
@@ -284,6 +295,7 @@ int copy_planes(ld_ctx* c, int z0, int nplanes, void* buf, bool pack, const char
     const size_t plane_bytes = (size_t)c->geom.nx * c->geom.ny * S;
     const size_t pitch_state = (size_t)c->geom.npad * S, pitch_buf = (size_t)nplanes * plane_bytes;
     char* state = static_cast<char*>(c->dist[c->cur]);
+    const bool local = on_one_device(buf, state);
     int rz[2], rn[2];
     const int runs = plane_runs(c, z0, nplanes, rz, rn);
     size_t done = 0;
@@ -291,10 +303,11 @@ int copy_planes(ld_ctx* c, int z0, int nplanes, void* buf, bool pack, const char
         char* st = state + (size_t)rz[r] * plane_bytes;
         char* bf = static_cast<char*>(buf) + done;
         const size_t width = (size_t)rn[r] * plane_bytes;
-        const cudaError_t e = pack ? cudaMemcpy2DAsync(bf, pitch_buf, st, pitch_state, width, 2 * kQ,
-                                                       cudaMemcpyDeviceToDevice, c->stream)
-                                   : cudaMemcpy2DAsync(st, pitch_state, bf, pitch_buf, width, 2 * kQ,
-                                                       cudaMemcpyDeviceToDevice, c->stream);
+        char *dst = pack ? bf : st, *from = pack ? st : bf;
+        const size_t dst_pitch = pack ? pitch_buf : pitch_state, from_pitch = pack ? pitch_state : pitch_buf;
+        const cudaError_t e = local ? ld::launch_copy_rows(dst, dst_pitch, from, from_pitch, width, 2 * kQ, c->stream)
+                                    : cudaMemcpy2DAsync(dst, dst_pitch, from, from_pitch, width, 2 * kQ,
+                                                        cudaMemcpyDeviceToDevice, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, where);
         done += width;
     }

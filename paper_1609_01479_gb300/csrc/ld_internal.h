@@ -127,6 +127,8 @@ cudaError_t launch_propagate(ld_ctx* c, int reverse);
 // uses for the mean of phi (the context's reduction scratch).
 cudaError_t launch_field_sum(ld_ctx* c, long long n, const double* x, double* out);
 cudaError_t launch_default_refs(ld_ctx* c);
+cudaError_t launch_copy_rows(void* dst, size_t dst_pitch, const void* src, size_t src_pitch, size_t bytes, int rows,
+                             cudaStream_t stream);
 
 // Raise a kernel's dynamic shared-memory limit to `bytes` on the current
 // device, once per device (the attribute belongs to the device's context).
