@@ -266,30 +266,25 @@ __global__ void __launch_bounds__(kAdjThreads)
 constexpr int kAdjFinalThreads = 1024;
 __global__ void __launch_bounds__(kAdjFinalThreads)
     k_adj_finalize(const double* __restrict__ part, int nkappa, int ntau, double taub_scale, double* __restrict__ grad) {
-    __shared__ double red[2][kAdjFinalThreads / 32];
+    // One block's sums run on one SM's FP64 pipe: a warp for each of the two
+    // adds the other warps' values (a shuffle tree in all 32 warps and a serial
+    // pass over them took 11 us).
+    __shared__ double red[2][kAdjFinalThreads];
     double a = 0.0, b = 0.0;
-    for (long long k = threadIdx.x; k < nkappa; k += kAdjFinalThreads) a += part[2 * k + 1];
-#pragma unroll 4
-    for (long long k = threadIdx.x; k < ntau; k += kAdjFinalThreads) b += part[2 * k];
-    for (int off = 16; off > 0; off >>= 1) {
-        a += __shfl_down_sync(0xffffffffu, a, off);
-        b += __shfl_down_sync(0xffffffffu, b, off);
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][warp] = a;
-        red[1][warp] = b;
-    }
+    for (int k = threadIdx.x; k < nkappa; k += kAdjFinalThreads) a += part[2 * (long long)k + 1];
+#pragma unroll 8
+    for (int k = threadIdx.x; k < ntau; k += kAdjFinalThreads) b += part[2 * (long long)k];
+    red[0][threadIdx.x] = a;
+    red[1][threadIdx.x] = b;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double ka = 0.0, tb = 0.0;
-        for (int w = 0; w < kAdjFinalThreads / 32; ++w) {
-            ka += red[0][w];
-            tb += red[1][w];
-        }
-        grad[0] += ka;
-        grad[1] += taub_scale * tb;
-    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp > 1) return;
+    double v[4] = {0.0, 0.0, 0.0, 0.0};  // four chains: the additions' latency, not their number, is what waits
+#pragma unroll
+    for (int w = 0; w < kAdjFinalThreads / 32; ++w) v[w & 3] += red[warp][lane + 32 * w];
+    double t = (v[0] + v[1]) + (v[2] + v[3]);
+    for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
+    if (lane == 0) grad[warp] += warp == 0 ? t : taub_scale * t;
 }
 
 // Seed: fbar = 0, gbar_i = phibar (the adjoint of phi_T = sum_i g_i), i.e.
