@@ -236,27 +236,70 @@ __device__ __forceinline__ void mu_diffs_of_phi(const RowGeom& rg, const Model<R
          chem_potential(zm, xpzm + xmzm + ypzm + ymzm + c + p[zm2], m);
 }
 
-// Whether the step's collision forms mu from phi itself (mu_diffs_of_phi) and
-// k_mu is not launched: with the 7-point stencils and the potential force,
-// except in FP64, where seven mu per site would add 60 FP64 instructions.
+// The force -div P (7-point stencils) and mu at a site from phi alone: the
+// components P_ab that the divergence reads at the six neighbours, each the
+// operations of k_stress, from the 25 phi within two sites.
+template <class R>
+__device__ __forceinline__ void stress_force_of_phi(const RowGeom& rg, const Model<R>& m, const R* phi, int x, int y,
+                                                    int z, int s, const RowNbr& o, R& mu, R& Fx, R& Fy, R& Fz) {
+    const int nx = rg.nx, plane = rg.nx * rg.ny;
+    const int x2 = x + 2 >= nx ? 2 - nx : 2, xm2 = x < 2 ? nx - 2 : -2;
+    const int y2 = (y + 2 >= rg.ny ? 2 - rg.ny : 2) * nx, ym2 = (y < 2 ? rg.ny - 2 : -2) * nx;
+    const int z2 = (z + 2 >= rg.nz ? 2 - rg.nz : 2) * plane, zm2 = (z < 2 ? rg.nz - 2 : -2) * plane;
+    const R* p = phi + s;
+    const R c = p[0], xp = p[o.xp], xm = p[o.xm], yp = p[o.yp], ym = p[o.ym], zp = p[o.zp], zm = p[o.zm];
+    const R xpyp = p[o.xp + o.yp], xpym = p[o.xp + o.ym], xmyp = p[o.xm + o.yp], xmym = p[o.xm + o.ym];
+    const R xpzp = p[o.xp + o.zp], xpzm = p[o.xp + o.zm], xmzp = p[o.xm + o.zp], xmzm = p[o.xm + o.zm];
+    const R ypzp = p[o.yp + o.zp], ypzm = p[o.yp + o.zm], ymzp = p[o.ym + o.zp], ymzm = p[o.ym + o.zm];
+    mu = chem_potential(c, xp + xm + yp + ym + zp + zm, m);
+    // P_xb, P_yb, P_zb (b the axis of the neighbour) from its phi and six neighbours
+    struct Col {
+        R x, y, z;
+    };
+    auto column = [&](int b, R ph, R pxp, R pxm, R pyp, R pym, R pzp, R pzm) {
+        const R gx = R(0.5) * (pxp - pxm), gy = R(0.5) * (pyp - pym), gz = R(0.5) * (pzp - pzm);
+        const R lap = pxp + pxm + pyp + pym + pzp + pzm - R(6) * ph;
+        const R pb = R(0.5) * m.A * ph * ph + R(0.75) * m.B * ph * ph * ph * ph;
+        const R iso = pb - m.kappa * ph * lap - R(0.5) * m.kappa * (gx * gx + gy * gy + gz * gz);
+        const R gb = b == 0 ? gx : (b == 1 ? gy : gz);
+        Col r{m.kappa * gx * gb, m.kappa * gy * gb, m.kappa * gz * gb};
+        (b == 0 ? r.x : (b == 1 ? r.y : r.z)) += iso;
+        return r;
+    };
+    const Col a = column(0, xp, p[x2], c, xpyp, xpym, xpzp, xpzm), b = column(0, xm, c, p[xm2], xmyp, xmym, xmzp, xmzm);
+    const Col d = column(1, yp, xpyp, xmyp, p[y2], c, ypzp, ypzm), e = column(1, ym, xpym, xmym, c, p[ym2], ymzp, ymzm);
+    const Col f = column(2, zp, xpzp, xmzp, ypzp, ymzp, p[z2], c), g = column(2, zm, xpzm, xmzm, ypzm, ymzm, c, p[zm2]);
+    Fx = -((R(0.5) * (a.x - b.x) + R(0.5) * (d.x - e.x)) + R(0.5) * (f.x - g.x));
+    Fy = -((R(0.5) * (a.y - b.y) + R(0.5) * (d.y - e.y)) + R(0.5) * (f.y - g.y));
+    Fz = -((R(0.5) * (a.z - b.z) + R(0.5) * (d.z - e.z)) + R(0.5) * (f.z - g.z));
+}
+
+// How the step's collision comes by mu and the force: from the fields that
+// k_mu or k_stress wrote (kFar), or from phi itself, without those launches:
+// kNearMu with the potential force, kNearStress with the stress force. The
+// near forms take the 7-point stencils (the 19-point ones would need 19 phi
+// at each of 18 neighbours) and FP32 arithmetic (in FP64 they would add 60 and
+// 200 instructions to the pipe that bounds the step).
+enum { kFar = 0, kNearMu = 1, kNearStress = 2 };
 template <int P>
-bool near_mu(const ld_ctx* c) {
-    return sizeof(typename Prec<P>::real_t) == 4 && !c->stress && c->prm.stencil == LD_STENCIL_7;
+int near_form(const ld_ctx* c) {
+    if (sizeof(typename Prec<P>::real_t) == 8 || c->prm.stencil != LD_STENCIL_7) return kFar;
+    return c->stress ? kNearStress : kNearMu;
 }
 
 // Resident blocks per SM the collision kernel is compiled for: 6 x 128
 // threads (80 registers) with FP32 arithmetic, 5 (96) where it forms mu from
 // phi, 3 with FP64.
-template <int P, bool NEAR>
+template <int P, int NEAR>
 constexpr int rows_blocks_per_sm() {
-    return sizeof(typename Prec<P>::real_t) == 4 ? (NEAR ? 5 : 6) : 3;
+    return sizeof(typename Prec<P>::real_t) == 4 ? (NEAR != kFar ? 5 : 6) : 3;
 }
 
 // Stage 3: force, velocity, collisions of f and g, and propagation (push: the
 // post-collision value of direction i goes to x + c_i) with streaming stores;
-// NEAR: mu and its gradient formed here from phi (mu_out, when not null,
-// receives mu); SR: the 16-bit stores rounded stochastically from `sr`.
-template <int P, class I, bool NEAR, bool SR>
+// NEAR: where mu and the force come from (near forms write mu to mu_out when
+// it is not null); SR: the 16-bit stores rounded stochastically from `sr`.
+template <int P, class I, int NEAR, bool SR>
 __global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
     k_collide(RowGeom rg, I npad, Model<typename Prec<P>::real_t> m, SrStream sr, const typename Prec<P>::store_t* __restrict__ fs,
               const typename Prec<P>::store_t* __restrict__ gs, typename Prec<P>::store_t* __restrict__ fd,
@@ -286,7 +329,10 @@ __global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
     const int oxp = o.xp, oxm = o.xm, oyp = o.yp, oym = o.ym, ozp = o.zp, ozm = o.zm;
     const R ph = phi[s];
     R muc, Fx, Fy, Fz;
-    if constexpr (NEAR) {
+    if constexpr (NEAR == kNearStress) {
+        stress_force_of_phi(rg, m, phi, x, y, z, s, o, muc, Fx, Fy, Fz);
+        if (mu_out) mu_out[s] = muc;
+    } else if constexpr (NEAR == kNearMu) {
         R dx, dy, dz;
         mu_diffs_of_phi(rg, m, phi, x, y, z, s, o, muc, dx, dy, dz);
         force_of_diffs(ph, dx, dy, dz, Fx, Fy, Fz);
@@ -831,22 +877,22 @@ cudaError_t phi_mu_p(ld_ctx* c, const void* state) {
 
 // One step; phi and mu of the source state go to `fields` ([phi npad][mu
 // npad]) when it is not null, else to the context's scratch.
-template <int P, class I, bool NEAR, bool SR>
+template <int P, class I, int NEAR, bool SR>
 cudaError_t collide_rows(ld_ctx* c, const void* src, void* dst, void* fields) {
     using S = typename Prec<P>::store_t;
     using R = typename Prec<P>::real_t;
     R* phi = fields ? (R*)fields : (R*)c->phi;
     R* mu = fields ? (R*)fields + c->geom.npad : (R*)c->mu;
     launch_phi<P, I>(c, src, phi);
-    if (!NEAR) launch_mu<R, I>(c, phi, mu);
+    if (NEAR == kFar) launch_mu<R, I>(c, phi, mu);
     k_collide<P, I, NEAR, SR><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
         row_geom(c->geom), (I)c->geom.npad, model_of<R>(c->prm), sr_stream(c->prm.seed, c->sr_step, c->geom.n),
         (const S*)f_part(c, src), (const S*)g_part(c, src), (S*)f_part(c, dst), (S*)g_part(c, dst), phi,
-        NEAR ? nullptr : mu, c->ref, (const R*)c->stress, NEAR && fields ? mu : nullptr, c->status);
+        NEAR != kFar ? nullptr : mu, c->ref, (const R*)c->stress, NEAR != kFar && fields ? mu : nullptr, c->status);
     return cudaGetLastError();
 }
 
-template <int P, bool NEAR, bool SR>
+template <int P, int NEAR, bool SR>
 cudaError_t collide_r(ld_ctx* c, const void* src, void* dst, void* fields) {
     return offsets_fit_int(c) ? collide_rows<P, int, NEAR, SR>(c, src, dst, fields)
                               : collide_rows<P, long long, NEAR, SR>(c, src, dst, fields);
@@ -855,9 +901,12 @@ cudaError_t collide_r(ld_ctx* c, const void* src, void* dst, void* fields) {
 template <int P, bool SR>
 cudaError_t collide_n(ld_ctx* c, const void* src, void* dst, void* fields) {
     if constexpr (sizeof(typename Prec<P>::real_t) == 4) {
-        if (near_mu<P>(c)) return collide_r<P, true, SR>(c, src, dst, fields);
+        switch (near_form<P>(c)) {
+            case kNearMu: return collide_r<P, kNearMu, SR>(c, src, dst, fields);
+            case kNearStress: return collide_r<P, kNearStress, SR>(c, src, dst, fields);
+        }
     }
-    return collide_r<P, false, SR>(c, src, dst, fields);
+    return collide_r<P, kFar, SR>(c, src, dst, fields);
 }
 
 template <int P>
