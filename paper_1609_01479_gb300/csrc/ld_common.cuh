@@ -37,23 +37,6 @@ __host__ __device__ constexpr R wgt(int i) {
 }
 
 // ---------------------------------------------------------------------------
-// x - y rounded to odd (Boldo & Melquiond 2008): the difference truncated
-// toward zero, with the last bit set where it is inexact. Rounding the
-// result to a format of at most 22 bits gives what rounding the exact
-// difference once would. The error of the float difference is exact (Knuth's
-// two-sum); truncated with the sticky bit, an inexact difference whose last
-// bit is clear moves by one unit, away from zero if the error has its sign,
-// else toward zero. Eight FP32 and integer operations instead of two
-// conversions and a subtraction on the FP64 pipe.
-__device__ __forceinline__ float sub_to_odd(float x, float y) {
-    const float d = __fsub_rn(x, y);
-    const float b = __fsub_rn(d, x);
-    const float e = __fsub_rn(__fsub_rn(x, __fsub_rn(d, b)), __fadd_rn(y, b));
-    const int u = __float_as_int(d), v = __float_as_int(e);
-    if (e == 0.0f || (u & 1) || !(fabsf(d) <= 3.4028234e38f)) return d;
-    return __int_as_float((u ^ v) < 0 ? u - 1 : u + 1);
-}
-
 // Storage precisions. real_t is the arithmetic type; store_t the stored one.
 // The 16-bit forms store the deviation from a per-direction reference value.
 // decode/encode work in real_t inside the step; decode_d/encode_d convert
@@ -89,7 +72,7 @@ template <> struct Prec<LD_FP16DEV> {
     __device__ static store_t encode_sr(float x, float ref, unsigned k);
     __device__ static double decode_d(store_t v, float ref) { return (double)ref + (double)__half2float(v); }
     __device__ static store_t encode_d(double x, float ref) { return __double2half(x - (double)ref); }
-    __device__ static store_t encode_r(float x, float ref) { return __float2half_rn(sub_to_odd(x, ref)); }
+    __device__ static store_t encode_r(float x, float ref);
 };
 template <> struct Prec<LD_BF16DEV> {
     using store_t = __nv_bfloat16;
@@ -100,8 +83,33 @@ template <> struct Prec<LD_BF16DEV> {
     __device__ static store_t encode_sr(float x, float ref, unsigned k);
     __device__ static double decode_d(store_t v, float ref) { return (double)ref + (double)__bfloat162float(v); }
     __device__ static store_t encode_d(double x, float ref) { return __double2bfloat16(x - (double)ref); }
-    __device__ static store_t encode_r(float x, float ref) { return __float2bfloat16_rn(sub_to_odd(x, ref)); }
+    __device__ static store_t encode_r(float x, float ref);
 };
+
+// encode_d of a float x with few instructions on the FP64 pipe, which bounded
+// the initialiser (38 differences and conversions a site). x - ref lies within
+// one unit of the float difference; where the floats one unit below and above
+// it round to the same 16-bit value, that is the value, and else (about one
+// value in 4000) the FP64 form decides. A call, so that the FP64 instructions
+// are not issued with a false predicate.
+template <int P>
+__device__ __noinline__ typename Prec<P>::store_t encode_d_call(float x, float ref) {
+    return Prec<P>::encode_d((double)x, ref);
+}
+__device__ __forceinline__ __half Prec<LD_FP16DEV>::encode_r(float x, float ref) {
+    const float d = __fsub_rn(x, ref);
+    const __half lo = __float2half_rn(__int_as_float(__float_as_int(d) - 1));
+    const __half hi = __float2half_rn(__int_as_float(__float_as_int(d) + 1));
+    if (d == 0.0f) return __float2half_rn(0.0f);
+    return __half_as_ushort(lo) == __half_as_ushort(hi) ? lo : encode_d_call<LD_FP16DEV>(x, ref);
+}
+__device__ __forceinline__ __nv_bfloat16 Prec<LD_BF16DEV>::encode_r(float x, float ref) {
+    const float d = __fsub_rn(x, ref);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(__int_as_float(__float_as_int(d) - 1));
+    const __nv_bfloat16 hi = __float2bfloat16_rn(__int_as_float(__float_as_int(d) + 1));
+    if (d == 0.0f) return __float2bfloat16_rn(0.0f);
+    return __bfloat16_as_ushort(lo) == __bfloat16_as_ushort(hi) ? lo : encode_d_call<LD_BF16DEV>(x, ref);
+}
 
 // Stochastic rounding of the FP32 deviation h to a 16-bit format with the
 // 16-bit random integer k (Connolly, Higham & Mary 2021, mode 1): lo = h
@@ -682,20 +690,25 @@ __device__ __forceinline__ void collide_f_trt(double (&f)[Q], double rho, double
 }
 
 // Equilibria of a site, feq_i and geq_i, handed to out(i, feq, geq): one
-// direction at a time in FP32; on opposite pairs with fused operations in FP64,
-// where 19 directions took about 330 instructions on the FP64 pipe.
+// direction at a time in FP32, every fusion of a product and a sum written out
+// (left to the compiler it changed with the code around it, and with it the
+// last bit of an initial state); on opposite pairs with fused operations in
+// FP64, where 19 directions took about 330 instructions on the FP64 pipe.
 template <class Out>
 __device__ __forceinline__ void equilibria(float rho, float p, float mu, float Gamma, float ux, float uy, float uz,
                                            Out out) {
     const float uu = ux * ux + uy * uy + uz * uz;
-    const float dev = Gamma * mu - p / 3.0f;
+    const float dev = Gamma * mu - p / 3.0f, dev45 = __fmul_rn(4.5f, dev);
+    const float p3 = __fmul_rn(3.0f, p), p45 = __fmul_rn(4.5f, p), mp15 = -__fmul_rn(1.5f, p);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
         const float cu = cdot(i, ux, uy, uz);
-        const float feq = wgt<float>(i) * rho * (1.0f + 3.0f * cu + 4.5f * cu * cu - 1.5f * uu);
-        const float geq = wgt<float>(i) * (p + 3.0f * p * cu + 4.5f * dev * float(c2(i) - 1) + 4.5f * p * cu * cu -
-                                           1.5f * p * uu);
-        out(i, feq, geq);
+        const float s = __fmaf_rn(-1.5f, uu, __fmaf_rn(__fmul_rn(4.5f, cu), cu, __fmaf_rn(3.0f, cu, 1.0f)));
+        float t = __fmaf_rn(p3, cu, p);
+        if (c2(i) == 2) t = __fadd_rn(t, dev45);
+        if (c2(i) == 0) t = __fsub_rn(t, dev45);
+        t = __fmaf_rn(mp15, uu, __fmaf_rn(__fmul_rn(p45, cu), cu, t));
+        out(i, __fmul_rn(__fmul_rn(wgt<float>(i), rho), s), __fmul_rn(wgt<float>(i), t));
     }
 }
 template <class Out>
