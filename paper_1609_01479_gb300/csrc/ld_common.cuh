@@ -118,28 +118,38 @@ __device__ __forceinline__ __nv_bfloat16 Prec<LD_BF16DEV>::encode_r(float x, flo
 // exact in FP32 (|hi| - |lo| is a power of two, |h| - |lo| is exact by
 // Sterbenz's lemma or because lo = 0), so the decision is a function of h and
 // k alone. Exact values, NaN and the largest finite magnitude are kept.
-__device__ __forceinline__ bool sr_up(float h, float lo, float hi, unsigned k) {
-    const float gap = __fsub_rn(fabsf(hi), fabsf(lo));
-    const float d = __fsub_rn(fabsf(h), fabsf(lo));
-    return __fmul_rn((float)k, gap) < __fmul_rn(d, 65536.0f);
-}
+// The 38 stores of a site make most of a step's instructions, so the spacing
+// |hi| - |lo| is formed from the exponent of h (at least 2^-14, below which
+// halves are 2^-24 apart), k becomes a float as the low bits of 2^23 + k, and
+// an exact value needs no test of its own (its right side is 0).
 __device__ __forceinline__ __half Prec<LD_FP16DEV>::encode_sr(float x, float ref, unsigned k) {
     const float h = x - ref;
     const __half lo = __float2half_rz(h);
-    const float lof = __half2float(lo);
-    const unsigned short b = __half_as_ushort(lo);
-    if (lof == h || (b & 0x7fffu) == 0x7bffu) return lo;
-    const __half hi = __ushort_as_half((unsigned short)(b + 1));
-    return sr_up(h, lof, __half2float(hi), k) ? hi : lo;
+    const unsigned b = __half_as_ushort(lo);
+    const float d = __fsub_rn(fabsf(h), fabsf(__half2float(lo)));
+    const int e = max(__float_as_int(h) & 0x7f800000, 113 << 23);
+    const float gap = __int_as_float(e - (10 << 23)), kf = __fsub_rn(__int_as_float(0x4b000000u | k), 8388608.0f);
+    const bool up = __fmul_rn(kf, gap) < __fmul_rn(d, 65536.0f) && (b & 0x7fffu) != 0x7bffu;
+    return __ushort_as_half((unsigned short)(b + (up ? 1u : 0u)));
 }
+// A bfloat16 is the upper half of the float's bits, its spacing the lower
+// half's range: hi is taken when k < the lower half. From 2^111 on, where the
+// products of the rule leave the range of floats, and for NaN, the rule as it
+// stands.
 __device__ __forceinline__ __nv_bfloat16 Prec<LD_BF16DEV>::encode_sr(float x, float ref, unsigned k) {
     const float h = x - ref;
-    const __nv_bfloat16 lo = __float2bfloat16_rz(h);
-    const float lof = __bfloat162float(lo);
-    const unsigned short b = __bfloat16_as_ushort(lo);
-    if (lof == h || (b & 0x7fffu) == 0x7f7fu) return lo;
-    const __nv_bfloat16 hi = __ushort_as_bfloat16((unsigned short)(b + 1));
-    return sr_up(h, lof, __bfloat162float(hi), k) ? hi : lo;
+    const unsigned u = __float_as_uint(h), b = u >> 16;
+    if ((u & 0x7fffffffu) >= 0x77000000u) {
+        const __nv_bfloat16 lo = __float2bfloat16_rz(h);
+        const unsigned c = __bfloat16_as_ushort(lo);
+        const float lof = __bfloat162float(lo);
+        if (lof == h || (c & 0x7fffu) == 0x7f7fu) return lo;
+        const float hif = __bfloat162float(__ushort_as_bfloat16((unsigned short)(c + 1)));
+        const float gap = __fsub_rn(fabsf(hif), fabsf(lof)), d = __fsub_rn(fabsf(h), fabsf(lof));
+        const bool up = __fmul_rn((float)k, gap) < __fmul_rn(d, 65536.0f);
+        return __ushort_as_bfloat16((unsigned short)(c + (up ? 1u : 0u)));
+    }
+    return __ushort_as_bfloat16((unsigned short)(b + (k < (u & 0xffffu) ? 1u : 0u)));
 }
 
 // Random words of stochastic rounding: SplitMix64 (Steele, Lea & Flood 2014)
