@@ -57,7 +57,8 @@ extern "C" {
 enum { LD_FP64 = 0, LD_FP32 = 1, LD_FP16DEV = 2, LD_BF16DEV = 3 };
 
 /* Step kernel selection.
- * LD_KERNEL_GENERIC: three launches per step (phi, mu, collide+propagate); any lattice.
+ * LD_KERNEL_GENERIC: launches in site order (phi, mu where the collision does not
+ *   form it from phi, collide+propagate); any lattice.
  * LD_KERNEL_FUSED: one launch per step that reads and writes each distribution
  *   once from HBM; phi and mu rings in shared memory, distributions through
  *   registers (nx % 32 == 0, ny % 8 == 0, nz % 4 == 0).

@@ -18,7 +18,7 @@
 // Each site sees the same operations as in collide_f_dev / collide_g_dev,
 // except that the packed forms fix where a product and a sum fuse (the
 // scalar kernel leaves that to the compiler); the results agree within FP32
-// rounding. Round to nearest only (stochastic rounding runs k_step_fused).
+// rounding. Either rounding of the stores (SR).
 // The same scheme for FP32 storage measured slower than k_step_fused (0.68 of
 // the HBM roofline at 384^3 against 0.74): FP32 is bound by memory latency
 // rather than by instructions, and two sites' values in registers leave a

@@ -1,7 +1,7 @@
 // Generic kernels: any lattice size >= 4 in every dimension, one thread per
-// site. The step runs as three launches in row order -- phi (zeroth moment
-// of g), mu (7- or 19-point Laplacian), and collide+propagate, with a fourth
-// for the chemical stress when the force is -div P -- and the same file holds the
+// site. The step runs as launches in site order -- phi (zeroth moment of g),
+// mu or the chemical stress where the collision does not form them from phi,
+// and collide+propagate -- and the same file holds the
 // initialiser, the macroscopic output, the FP64 conservation sums, the
 // codec I/O and propagation alone. Templates only: instantiated per storage
 // precision by ld_prec_f64.cu and ld_prec_lp.cu.

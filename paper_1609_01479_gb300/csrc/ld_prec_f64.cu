@@ -1,7 +1,7 @@
-// FP64 instantiation of the step kernels. Built with -fmad=false: every
-// product and sum rounds separately (no fused multiply-add contraction), in
-// the operation order each kernel writes -- the formulas' own order, or the
-// opposite-pair forms of the collisions (ld_common.cuh).
+// FP64 instantiation of the step kernels. Built with -fmad=false: the compiler
+// contracts nothing, products and sums fuse only where a kernel writes
+// __fma_rn (the opposite-pair forms of the collisions, ld_common.cuh), so every
+// kernel that shares a helper gets the same bits.
 #include "ld_fused.cuh"
 #include "ld_generic.cuh"
 #include "ld_adjoint.cuh"
