@@ -118,15 +118,20 @@ bool is_device_ptr(const void* p) {
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Whether both pointers are device memory of one GPU (the copy kernel cannot
-// reach another GPU's memory, the runtime's copies can).
-bool on_one_device(const void* p, const void* q) {
+// Whether a copy between p and q may run as the copy kernel: both are device
+// memory of the current GPU. A kernel is launched on that GPU and would reach
+// another's memory only by chance of peer access; the runtime's copies serve a
+// context of any GPU whichever is current.
+bool copy_kernel_reaches(const void* p, const void* q) {
     cudaPointerAttributes a, b;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, q) != cudaSuccess) {
+    int current = 0;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaPointerGetAttributes(&b, q) != cudaSuccess ||
+        cudaGetDevice(&current) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return a.type == cudaMemoryTypeDevice && b.type == cudaMemoryTypeDevice && a.device == b.device;
+    return a.type == cudaMemoryTypeDevice && b.type == cudaMemoryTypeDevice && a.device == current &&
+           b.device == current;
 }
 
 bool opt_device(const void* p) { return p == nullptr || is_device_ptr(p); }
@@ -295,7 +300,7 @@ int copy_planes(ld_ctx* c, int z0, int nplanes, void* buf, bool pack, const char
     const size_t plane_bytes = (size_t)c->geom.nx * c->geom.ny * S;
     const size_t pitch_state = (size_t)c->geom.npad * S, pitch_buf = (size_t)nplanes * plane_bytes;
     char* state = static_cast<char*>(c->dist[c->cur]);
-    const bool local = on_one_device(buf, state);
+    const bool local = copy_kernel_reaches(buf, state);
     int rz[2], rn[2];
     const int runs = plane_runs(c, z0, nplanes, rz, rn);
     size_t done = 0;
@@ -305,9 +310,12 @@ int copy_planes(ld_ctx* c, int z0, int nplanes, void* buf, bool pack, const char
         const size_t width = (size_t)rn[r] * plane_bytes;
         char *dst = pack ? bf : st, *from = pack ? st : bf;
         const size_t dst_pitch = pack ? pitch_buf : pitch_state, from_pitch = pack ? pitch_state : pitch_buf;
-        const cudaError_t e = local ? ld::launch_copy_rows(dst, dst_pitch, from, from_pitch, width, 2 * kQ, c->stream)
-                                    : cudaMemcpy2DAsync(dst, dst_pitch, from, from_pitch, width, 2 * kQ,
-                                                        cudaMemcpyDeviceToDevice, c->stream);
+        // a launch on another GPU's stream is refused, a runtime copy is not (asking for a stream's
+        // GPU beforehand would end a capture)
+        cudaError_t e = cudaErrorInvalidResourceHandle;
+        if (local) e = ld::launch_copy_rows(dst, dst_pitch, from, from_pitch, width, 2 * kQ, c->stream);
+        if (e == cudaErrorInvalidResourceHandle)
+            e = cudaMemcpy2DAsync(dst, dst_pitch, from, from_pitch, width, 2 * kQ, cudaMemcpyDeviceToDevice, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, where);
         done += width;
     }

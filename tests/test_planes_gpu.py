@@ -37,3 +37,27 @@ def test_planes_survive_the_round_trip(precision, dims, offset):
         assert torch.equal(after[:, idx], state[:, idx])
         rest = [z for z in range(nz) if z not in idx]
         assert torch.equal(after[:, rest], before[:, rest])
+
+
+def test_planes_in_a_graph():
+    """Both copies under stream capture, on a stream of their own; a replay copies the state of its time."""
+    nx, ny, nz = 9, 5, 8
+    sim = ld.LdSim(nx, ny, nz, precision="fp32")
+    stream = torch.cuda.Stream()
+    ld.ld_set_stream(sim.ctx, stream.cuda_stream)
+    f, g = torch.rand((2, 19, nz, ny, nx), dtype=torch.float64, device="cuda")
+    buf = torch.empty((38, 2, ny, nx), dtype=torch.float32, device="cuda")
+    stream.wait_stream(torch.cuda.current_stream())
+    sim.set_distributions(f, g)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        ld.ld_pack_planes(sim.ctx, 1, 2, buf)
+        ld.ld_unpack_planes(sim.ctx, 5, 2, buf)
+    with torch.cuda.stream(stream):
+        sim.set_distributions(g, f)
+        graph.replay()
+        after = torch.cat(sim.distributions())
+    stream.synchronize()
+    want = torch.cat((g, f)).float().double()
+    want[:, 5:7] = want[:, 1:3]
+    assert torch.equal(after, want)
