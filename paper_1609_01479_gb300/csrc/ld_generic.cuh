@@ -731,6 +731,16 @@ __device__ __forceinline__ bool macros_site(const MacrosArgs<P>& a, unsigned s, 
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) u[c] = div_by(num[c], rho, inv);
+        if constexpr (!FAST) {  // (FAST takes only densities within the range of floats)
+            if (__builtin_expect(any_nonfinite(u[0], u[1], u[2]), 0)) {
+                // j is the sum of c_i f_i over every i: an infinite f_i leaves no component of it a value
+                double z = 0.0;
+#pragma unroll 1
+                for (int i = 0; i < Q; ++i) z = __fma_rn(0.0, Prec<P>::decode_d(a.fs[i * npad + s], ref[i]), z);
+#pragma unroll
+                for (int c = 0; c < 3; ++c) u[c] = z == 0.0 ? __ddiv_rn(num[c], rho) : z;
+            }
+        }
     }
     if (a.gphi_out) grad(a.phi, gp);
     if (FAST && !ok) return false;
