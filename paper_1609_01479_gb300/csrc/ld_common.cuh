@@ -98,16 +98,16 @@ __device__ __noinline__ typename Prec<P>::store_t encode_d_call(float x, float r
 }
 __device__ __forceinline__ __half Prec<LD_FP16DEV>::encode_r(float x, float ref) {
     const float d = __fsub_rn(x, ref);
-    const __half lo = __float2half_rn(__int_as_float(__float_as_int(d) - 1));
-    const __half hi = __float2half_rn(__int_as_float(__float_as_int(d) + 1));
-    if (d == 0.0f) return __float2half_rn(0.0f);
+    const __half lo = __float2half_rn(__uint_as_float(__float_as_uint(d) - 1));
+    const __half hi = __float2half_rn(__uint_as_float(__float_as_uint(d) + 1));
+    if (d == 0.0f) return __float2half_rn(d);  // with its sign
     return __half_as_ushort(lo) == __half_as_ushort(hi) ? lo : encode_d_call<LD_FP16DEV>(x, ref);
 }
 __device__ __forceinline__ __nv_bfloat16 Prec<LD_BF16DEV>::encode_r(float x, float ref) {
     const float d = __fsub_rn(x, ref);
-    const __nv_bfloat16 lo = __float2bfloat16_rn(__int_as_float(__float_as_int(d) - 1));
-    const __nv_bfloat16 hi = __float2bfloat16_rn(__int_as_float(__float_as_int(d) + 1));
-    if (d == 0.0f) return __float2bfloat16_rn(0.0f);
+    const __nv_bfloat16 lo = __float2bfloat16_rn(__uint_as_float(__float_as_uint(d) - 1));
+    const __nv_bfloat16 hi = __float2bfloat16_rn(__uint_as_float(__float_as_uint(d) + 1));
+    if (d == 0.0f) return __float2bfloat16_rn(d);  // with its sign
     return __bfloat16_as_ushort(lo) == __bfloat16_as_ushort(hi) ? lo : encode_d_call<LD_BF16DEV>(x, ref);
 }
 

@@ -114,3 +114,17 @@ def test_totals_of_sizes_off_the_vectors(precision, dims):
     tol = 20 * unit * np.array([np.abs(f).sum(), np.abs(g).sum()]) + n * 2.0 ** -52
     assert (np.abs(got[:2] - want) <= tol).all()
     assert np.abs(got[2:]).max() <= 20 * unit * np.abs(f).sum()
+
+
+@pytest.mark.parametrize("precision", ["fp16dev", "bf16dev"])
+def test_initial_zeros_keep_their_sign(precision):
+    """phi = +-2^-149 with mean 0: the references are 0 and w_i phi along the axes underflows to a zero with phi's
+    sign, which the deviation of the FP64 form, x - 0, keeps."""
+    nx, ny, nz = 10, 6, 5
+    phi = np.full(nx * ny * nz, 2.0 ** -149)
+    phi[1::2] *= -1.0
+    phi = phi.reshape(nz, ny, nx)
+    sim = ld.LdSim(nx, ny, nz, precision=precision)
+    sim.init(torch.from_numpy(phi))
+    bits = planes(sim, precision)[20:26].view(torch.int16).cpu().numpy().view(np.uint16)
+    assert np.array_equal(bits, np.broadcast_to(np.where(phi < 0, 0x8000, 0).astype(np.uint16), bits.shape))
