@@ -101,6 +101,13 @@ bool params_ok(const ld_params* p, const char** why) {
     return true;
 }
 
+// The stress form of the force and the TRT collision run on the generic kernel.
+int step_kernel_of(int nx, int ny, int nz, const ld_params& p) {
+    return p.force == LD_FORCE_STRESS || p.collision == LD_COLLISION_TRT
+               ? ld::kStepGeneric
+               : ld::choose_step_kernel(nx, ny, nz, p.precision, p.stencil, p.kernel);
+}
+
 bool dims_ok(int nx, int ny, int nz) {
     if (nx < 4 || ny < 4 || nz < 4) return false;
     // every index and offset fits the 64-bit arithmetic; keep n within 2^31 sites
@@ -178,10 +185,7 @@ int ld_create(int nx, int ny, int nz, const ld_params* p, void* dev_workspace, s
     if ((uintptr_t)dev_workspace % kAlign) return fail(nullptr, LD_EINVAL, "workspace must be 256-byte aligned");
     if (bytes < L.total)
         return fail(nullptr, LD_EINVAL, "workspace of %zu bytes is smaller than the %zu needed", bytes, L.total);
-    // the stress form of the force and the TRT collision run on the generic kernel
-    const int step_kernel = p->force == LD_FORCE_STRESS || p->collision == LD_COLLISION_TRT
-                                ? ld::kStepGeneric
-                                : ld::choose_step_kernel(nx, ny, nz, p->precision, p->kernel);
+    const int step_kernel = step_kernel_of(nx, ny, nz, *p);
     if (step_kernel == 0)
         return fail(nullptr, LD_EINVAL,
                     "fused kernels need nx %% 32 == 0, ny %% 8 == 0, nz %% 4 == 0 (staged: FP32/FP16DEV/BF16DEV only)");
@@ -256,6 +260,7 @@ int ld_set_params(ld_ctx* c, const ld_params* p) {
         return fail(c, LD_EINVAL,
                     "precision, kernel, rho0, the force form, the collision and the rounding are fixed at ld_create");
     c->prm = *p;
+    c->step_kernel = step_kernel_of(c->geom.nx, c->geom.ny, c->geom.nz, *p);
     return LD_OK;
 }
 
@@ -381,7 +386,7 @@ int ld_step_kernel(const ld_ctx* c) {
         case ld::kStepStaged: return LD_KERNEL_FUSED_STAGED;
         // AUTO on a small lattice, whose one launch does the step of either
         case ld::kStepSmall:
-            return ld::choose_step_kernel(c->geom.nx, c->geom.ny, c->geom.nz, c->prec, LD_KERNEL_FUSED)
+            return ld::choose_step_kernel(c->geom.nx, c->geom.ny, c->geom.nz, c->prec, c->prm.stencil, LD_KERNEL_FUSED)
                        ? LD_KERNEL_FUSED
                        : LD_KERNEL_GENERIC;
         default: return LD_EINVAL;

@@ -148,9 +148,9 @@ cudaError_t set_max_dynamic_smem_once(int bytes) {
 
 // Step kernels (ld_ctx::step_kernel).
 enum StepKernel { kStepGeneric = 1, kStepStaged = 2, kStepRegs = 3, kStepSmall = 4 };
-// The kernel a request resolves to for this lattice and precision, or 0 if
-// the requested one cannot run it.
-int choose_step_kernel(int nx, int ny, int nz, int prec, int requested);
+// The kernel a request resolves to for this lattice, precision and stencil, or
+// 0 if the requested one cannot run it.
+int choose_step_kernel(int nx, int ny, int nz, int prec, int stencil, int requested);
 
 inline bool is_f64(const ld_ctx* c) { return c->prec == LD_FP64; }
 // ref_mean: host pointer to the mean phi the 16-bit forms' g references are

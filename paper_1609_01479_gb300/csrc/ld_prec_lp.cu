@@ -123,7 +123,7 @@ cudaError_t launch_field_sum(ld_ctx* c, long long n, const double* x, double* ou
     return cudaGetLastError();
 }
 cudaError_t launch_default_refs(ld_ctx* c) { return default_refs(c); }
-int choose_step_kernel(int nx, int ny, int nz, int prec, int requested) {
+int choose_step_kernel(int nx, int ny, int nz, int prec, int stencil, int requested) {
     const bool f64p = prec == LD_FP64;
     const bool staged = f64p ? f64::staged_supported(nx, ny, nz, prec) : lp::staged_supported(nx, ny, nz, prec);
     const bool regs = f64p ? f64::regs_supported(nx, ny, nz) : lp::regs_supported(nx, ny, nz);
@@ -131,10 +131,11 @@ int choose_step_kernel(int nx, int ny, int nz, int prec, int requested) {
         case LD_KERNEL_GENERIC: return kStepGeneric;
         case LD_KERNEL_FUSED: return regs ? kStepRegs : 0;
         case LD_KERNEL_FUSED_STAGED: return staged ? kStepStaged : 0;
-        // FP64 is bound by the FP64 pipe, and the three row-ordered launches
-        // do less FP64 work per site than the fused step (no halo phi sums)
+        // FP64 is bound by the FP64 pipe, and the site-ordered launches (three
+        // in FP64) do less FP64 work per site than the fused step (no halo phi
+        // sums)
         case LD_KERNEL_AUTO:
-            if (prec == LD_FP32 && small_supported_impl(nx, ny, nz)) return kStepSmall;
+            if (prec == LD_FP32 && small_supported_impl(nx, ny, nz, stencil, regs)) return kStepSmall;
             return regs && !f64p ? kStepRegs : kStepGeneric;
         default: return 0;
     }

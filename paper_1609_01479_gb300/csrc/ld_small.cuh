@@ -4,15 +4,15 @@
 // A lattice of a few hundred thousand sites lives in L2, and its step is bound
 // by latency: the z-marching kernel (ld_fused.cuh) gives a 32^3 lattice 32 CTAs
 // for 152 SMs, each of them eight planes of dependent phases, and the
-// row-ordered launches of other sizes three launches a step. Here a CTA of 256
+// site-ordered launches of other sizes two or three launches a step. Here a CTA of 256
 // threads owns a tile of 32 x 4 x 2 sites and runs three phases, each once:
 //   1. all loads at once: the thread's own f and g, and the g of the tile's
 //      2-site halo, summed to phi in shared memory;
 //   2. mu over the tile and its 1-site halo;
 //   3. force, collisions and push of the thread's site.
-// The phi sums of the halo are repeated between CTAs (about four sites of g
-// read from L2 per site), which costs bandwidth that a lattice of this size
-// does not use. Any lattice size: tiles may reach past the lattice, and the
+// The phi sums of the halo are repeated between CTAs (4.1 sites of g per site
+// with the 7-point stencils, 5.8 with the 19-point ones, from L2), which costs
+// bandwidth that a lattice of this size does not use. Any lattice size: tiles may reach past the lattice, and the
 // halo wraps any number of times.
 // Consecutive steps overlap their launches: each launch lets the next one
 // start its CTAs at once (programmatic dependent launch), which compute their
@@ -235,12 +235,34 @@ inline cudaError_t launch_small(ld_ctx* c, const void* src, void* dst, void* fie
 
 }  // namespace
 
-// Lattices that LD_KERNEL_AUTO gives to k_step_small: up to 2^18 sites, where
-// the repeated halo sums cost less than the other kernels' latency. Measured,
-// us a step against the kernel AUTO takes otherwise (z-marching where the
-// lattice is tiled, else the row launches): 24^3 5.2 (12.4), 32^3 5.9 (14.5), 48
-// x 40 x 36 9.8 (16.4), 50 x 61 x 47 17.1 (19.6), 64^3 21.6 (22.7), 96 x 64 x 64
-// 41.8 (32.5).
-inline bool small_supported_impl(int nx, int ny, int nz) { return (long long)nx * ny * nz <= 1 << 18; }
+// Lattices that LD_KERNEL_AUTO gives to k_step_small, by its tiles of 32 x 4 x 2
+// sites: a tile costs about the same however many of its sites are the
+// lattice's, so a lattice 4 sites wide pays for 8 times its own. Up to 304 tiles
+// (two CTAs per SM) are one wave; beyond it the time grows by a wave of 3 to 5
+// us, while the other kernels start from two launches (8.3 us, three with the
+// 19-point stencils 12.4 to 14.4) or from the z-march's chunk (15 to 17 us) and
+// stay there to some 30k to 130k sites. The lines lie where 223 measured
+// lattices of 1k to 512k sites, 4 to 1000 wide, put them, us a step of this
+// kernel and of the one AUTO takes otherwise:
+//   row launches, 7-point   20 x 57 x 57, 435 tiles: 8.6, 10.3; 4 x 64 x 64, 512:
+//     9.7, 8.3; 33 x 45 x 44, 528: 12.0, 10.3; 64 x 45 x 45, 552: 12.3, 12.4;
+//     50 x 61 x 47, 768: 17.1, 14.4; 33 x 63 x 63, 1024: 20.0, 14.2; 4 x 128 x 128,
+//     2048: 31, 10. From 448 tiles on it also depends on how full they are
+//     (n/432): 31 x 65 x 65, 561: 12.2, 13.9; 60^3, 900: 19.7, 20.6.
+//   row launches, 19-point  45^3, 552: 15.0, 16.5; 48 x 52 x 52, 676: 17.6, 18.6;
+//     50 x 61 x 47, 768: 20.4, 18.5; 33 x 65 x 65, 1122: 25.9, 18.5
+//   z-march, 7-point        32^3, 128: 5.9, 14.5; 96 x 96 x 24, 864: 19.5, 22.7;
+//     64^3, 1024: 23.0, 22.7; 32 x 128 x 64, 1024: 22.3, 20.7; 19-point 96 x 96 x 24:
+//     23.2, 24.7; 64^3: 26.6, 24.7
+// The choice costs at most 10 % against the faster kernel on any of them and of
+// 110 others, 0.1 to 0.2 % on average; by sites alone (up to 2^18) it cost up to
+// a factor of 5.8, 7 % on average of the 110.
+inline bool small_supported_impl(int nx, int ny, int nz, int stencil, bool tiled) {
+    const long long n = (long long)nx * ny * nz;
+    const long long tiles = (long long)((nx + kSmX - 1) / kSmX) * ((ny + kSmY - 1) / kSmY) * ((nz + kSmZ - 1) / kSmZ);
+    if (tiled) return tiles <= 912;
+    if (stencil == LD_STENCIL_19) return tiles <= 704;
+    return tiles <= 448 || tiles <= 300 + n / 432;
+}
 
 }  // namespace ld

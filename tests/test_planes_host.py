@@ -45,7 +45,7 @@ cudaError_t launch_copy_rows(void*, size_t, const void*, size_t, size_t, int, cu
     return ++g_kernel, cudaSuccess;
 }
 cudaError_t launch_default_refs(ld_ctx*) { return cudaSuccess; }
-int choose_step_kernel(int, int, int, int, int) { return kStepGeneric; }
+int choose_step_kernel(int, int, int, int, int, int) { return kStepGeneric; }
 namespace lp {
 cudaError_t init(ld_ctx*, const double*, const double*, const double*, const double*) { return cudaSuccess; }
 }
