@@ -753,7 +753,13 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_init(LcGeom g, double rho0, c
     if (s >= g.n) return;
     const T r = rho ? (T)rho[s] : (T)rho0;
     const T ux = uin ? (T)uin[s] : T(0), uy = uin ? (T)uin[g.n + s] : T(0), uz = uin ? (T)uin[2 * g.n + s] : T(0);
-    ld::equilibria(r, T(0), T(0), T(0), ux, uy, uz, [&](int i, T feq, T) { f[i * g.npad + s] = feq; });
+    // FP32 adds the squares in the order the crystal's initial states have had (init_uu starts with ux's)
+    T uu;
+    if constexpr (sizeof(T) == 4)
+        uu = ld::init_uu(uy, ux, uz);
+    else
+        uu = ld::init_uu(ux, uy, uz);
+    ld::equilibria(r, T(0), T(0), T(0), ux, uy, uz, uu, [&](int i, T feq, T) { f[i * g.npad + s] = feq; });
 #pragma unroll
     for (int k = 0; k < 5; ++k) q[k * g.npad + s] = (T)qin[k * g.n + s];
 }

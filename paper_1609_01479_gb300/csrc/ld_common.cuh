@@ -713,16 +713,28 @@ __device__ __forceinline__ void collide_f_trt(double (&f)[Q], double rho, double
     collide_f_pairs<true>(f, rho, ux, uy, uz, Fx, Fy, Fz, m.omega_f, m.pc);
 }
 
-// Equilibria of a site, feq_i and geq_i, handed to out(i, feq, geq): one
-// direction at a time in FP32, every fusion of a product and a sum written out
-// (left to the compiler it changed with the code around it, and with it the
-// last bit of an initial state); on opposite pairs with fused operations in
-// FP64, where 19 directions took about 330 instructions on the FP64 pipe.
+// a b + c of the initial state's mu: one rounding in FP32, two in FP64.
+__device__ __forceinline__ float init_mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double init_mad(double a, double b, double c) { return __dadd_rn(__dmul_rn(a, b), c); }
+
+// u.u of an initial state.
+__device__ __forceinline__ float init_uu(float ux, float uy, float uz) {
+    return __fmaf_rn(uz, uz, __fmaf_rn(ux, ux, __fmul_rn(uy, uy)));
+}
+__device__ __forceinline__ double init_uu(double ux, double uy, double uz) {
+    return __fma_rn(ux, ux, __fma_rn(uy, uy, __dmul_rn(uz, uz)));
+}
+
+// Equilibria of a site, feq_i and geq_i, handed to out(i, feq, geq), with uu
+// = u.u: one direction at a time in FP32, every fusion of a product and a sum
+// written out (left to the compiler it changed with the code around it, and
+// with it the last bit of an initial state); on opposite pairs with fused
+// operations in FP64, where 19 directions took about 330 instructions on the
+// FP64 pipe.
 template <class Out>
 __device__ __forceinline__ void equilibria(float rho, float p, float mu, float Gamma, float ux, float uy, float uz,
-                                           Out out) {
-    const float uu = ux * ux + uy * uy + uz * uz;
-    const float dev = Gamma * mu - p / 3.0f, dev45 = __fmul_rn(4.5f, dev);
+                                           float uu, Out out) {
+    const float dev = __fmaf_rn(Gamma, mu, -__fdiv_rn(p, 3.0f)), dev45 = __fmul_rn(4.5f, dev);
     const float p3 = __fmul_rn(3.0f, p), p45 = __fmul_rn(4.5f, p), mp15 = -__fmul_rn(1.5f, p);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -737,8 +749,7 @@ __device__ __forceinline__ void equilibria(float rho, float p, float mu, float G
 }
 template <class Out>
 __device__ __forceinline__ void equilibria(double rho, double p, double mu, double Gamma, double ux, double uy,
-                                           double uz, Out out) {
-    const double uu = __fma_rn(ux, ux, __fma_rn(uy, uy, __dmul_rn(uz, uz)));
+                                           double uz, double uu, Out out) {
     const double base = __fma_rn(-1.5, uu, 1.0);
     const double dev45 = 4.5 * __fma_rn(Gamma, mu, (-1.0 / 3.0) * p);
     const double rb = rho * base, pb = p * base;

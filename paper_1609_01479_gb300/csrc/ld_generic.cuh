@@ -411,15 +411,17 @@ __global__ void __launch_bounds__(kThreads)
         lap = R(0);
 #pragma unroll
         for (int i = 1; i < Q; ++i)
-            lap += lap19_coef<R>(i) *
-                   ((R)phi[site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny), step_coord(z, cz(i), g.nz))] -
-                    p);
+            lap = init_mad(
+                lap19_coef<R>(i),
+                (R)phi[site_of(g, step_coord(x, cx(i), g.nx), step_coord(y, cy(i), g.ny), step_coord(z, cz(i), g.nz))] - p,
+                lap);
     } else {
         lap = (R)phi[site_of(g, wrap_inc(x, g.nx), y, z)] + (R)phi[site_of(g, wrap_dec(x, g.nx), y, z)]
             + (R)phi[site_of(g, x, wrap_inc(y, g.ny), z)] + (R)phi[site_of(g, x, wrap_dec(y, g.ny), z)]
-            + (R)phi[site_of(g, x, y, wrap_inc(z, g.nz))] + (R)phi[site_of(g, x, y, wrap_dec(z, g.nz))] - R(6) * p;
+            + (R)phi[site_of(g, x, y, wrap_inc(z, g.nz))] + (R)phi[site_of(g, x, y, wrap_dec(z, g.nz))];
+        lap = init_mad(R(-6), p, lap);
     }
-    const R mu = m.A * p + m.B * p * p * p - m.kappa * lap;
+    const R mu = init_mad(-m.kappa, lap, init_mad(m.A, p, m.B * p * p * p));
     const R rho = (R)(rho_in ? rho_in[s] : rho0);
     R ux = R(0), uy = R(0), uz = R(0);
     if (u_in) {
@@ -427,7 +429,7 @@ __global__ void __launch_bounds__(kThreads)
         uy = (R)u_in[g.n + s];
         uz = (R)u_in[2 * g.n + s];
     }
-    equilibria(rho, p, mu, m.Gamma, ux, uy, uz, [&](int i, R feq, R geq) {
+    equilibria(rho, p, mu, m.Gamma, ux, uy, uz, init_uu(ux, uy, uz), [&](int i, R feq, R geq) {
         fd[i * g.npad + s] = Prec<P>::encode_r(feq, ref[i]);
         gd[i * g.npad + s] = Prec<P>::encode_r(geq, ref[Q + i]);
     });

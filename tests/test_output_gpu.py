@@ -128,3 +128,83 @@ def test_initial_zeros_keep_their_sign(precision):
     sim.init(torch.from_numpy(phi))
     bits = planes(sim, precision)[20:26].view(torch.int16).cpu().numpy().view(np.uint16)
     assert np.array_equal(bits, np.broadcast_to(np.where(phi < 0, 0x8000, 0).astype(np.uint16), bits.shape))
+
+
+def fma32(a, b, c):
+    """float32 a b + c with one rounding: the exact product's float64 sum rounded to odd, then to float32."""
+    p, c = a.astype(np.float64) * b, np.asarray(c, np.float64)
+    s = p + c
+    t = s - p
+    err = (p - (s - t)) + (c - t)
+    odd = (s.view(np.int64) & 1).astype(bool)
+    s = np.where((err != 0) & ~odd, np.nextafter(s, np.copysign(np.inf, err)), s)
+    return s.astype(np.float32)
+
+
+C = [(0, 0, 0), (1, 0, 0), (-1, 0, 0), (0, 1, 0), (0, -1, 0), (0, 0, 1), (0, 0, -1), (1, 1, 0), (-1, -1, 0), (1, -1, 0),
+     (-1, 1, 0), (1, 0, 1), (-1, 0, -1), (1, 0, -1), (-1, 0, 1), (0, 1, 1), (0, -1, -1), (0, 1, -1), (0, -1, 1)]
+
+
+def f32(v, like):
+    return np.full_like(like, np.float32(v))
+
+
+def dot(c, u):
+    cu = np.zeros_like(u[0])
+    for k, v in zip(c, u):
+        cu = cu + v if k > 0 else cu - v if k < 0 else cu
+    return cu
+
+
+def feq32(i, rho, u, uu):
+    cu = dot(C[i], u)
+    w = np.float32(1) / np.float32(3 if i == 0 else 18 if i <= 6 else 36)
+    return (w * rho) * fma32(f32(-1.5, uu), uu, fma32(np.float32(4.5) * cu, cu, fma32(f32(3, cu), cu, f32(1, cu))))
+
+
+@pytest.mark.parametrize("stencil", [7, 19])
+def test_fp32_initial_state_has_the_written_fusions(stencil):
+    """Bit for bit feq and geq with one rounding where the code says so, mu of phi included."""
+    nx, ny, nz = 13, 7, 6
+    rng = np.random.default_rng(12)
+    phi, rho = 0.4 * rng.standard_normal((nz, ny, nx)), 1.0 + 0.05 * rng.standard_normal((nz, ny, nx))
+    u = 0.05 * rng.standard_normal((3, nz, ny, nx))
+    prm = dict(A=-0.07, B=0.051, kappa=0.043, Gamma=0.37)
+    sim = ld.LdSim(nx, ny, nz, precision="fp32", stencil=stencil, **prm)
+    sim.init(*(torch.from_numpy(a) for a in (phi, rho, u)))
+    got = planes(sim, "fp32").cpu().numpy()
+    A, B, kappa, Gamma = (np.float32(prm[k]) for k in ("A", "B", "kappa", "Gamma"))
+    p, rho, u = phi.astype(np.float32), rho.astype(np.float32), u.astype(np.float32)
+    at = lambda c: np.roll(p, (-c[2], -c[1], -c[0]), (0, 1, 2))  # noqa: E731
+    if stencil == 7:
+        lap = at(C[1])
+        for i in range(2, 7):
+            lap = lap + at(C[i])
+        lap = fma32(f32(-6, p), p, lap)
+    else:
+        lap = np.zeros_like(p)
+        for i in range(1, 19):
+            lap = fma32(np.float32(1) / f32(3 if i <= 6 else 6, p), at(C[i]) - p, lap)
+    mu = fma32(f32(-kappa, p), lap, fma32(f32(A, p), p, B * p * p * p))
+    uu = fma32(u[2], u[2], fma32(u[0], u[0], u[1] * u[1]))
+    dev45 = np.float32(4.5) * fma32(f32(Gamma, p), mu, -(p / np.float32(3)))
+    for i in range(19):
+        cu, w = dot(C[i], u), np.float32(1) / np.float32(3 if i == 0 else 18 if i <= 6 else 36)
+        t = fma32(np.float32(3) * p, cu, p)
+        t = t + dev45 if i > 6 else t - dev45 if i == 0 else t
+        t = fma32(-(np.float32(1.5) * p), uu, fma32((np.float32(4.5) * p) * cu, cu, t))
+        assert np.array_equal(got[i], feq32(i, rho, u, uu)) and np.array_equal(got[19 + i], w * t)
+
+
+def test_fp32_crystal_initial_state_has_the_written_fusions():
+    nx, ny, nz = 13, 7, 6
+    rng = np.random.default_rng(13)
+    q, rho = 0.2 * rng.standard_normal((5, nz, ny, nx)), 1.0 + 0.05 * rng.standard_normal((nz, ny, nx))
+    u = 0.05 * rng.standard_normal((3, nz, ny, nx))
+    sim = ld.LcSim(nx, ny, nz, precision="fp32")
+    sim.init(*(torch.from_numpy(a) for a in (q, rho, u)))
+    got = sim.fields()["f"].cpu().numpy()
+    rho, u = rho.astype(np.float32), u.astype(np.float32)
+    uu = fma32(u[2], u[2], fma32(u[1], u[1], u[0] * u[0]))
+    for i in range(19):
+        assert np.array_equal(got[i], feq32(i, rho, u, uu).astype(np.float64))
