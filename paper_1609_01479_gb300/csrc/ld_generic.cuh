@@ -212,17 +212,26 @@ __device__ __forceinline__ void stress_force_at(int iso, const T* P, I npad, int
     Fz = -((d[4][0] + d[5][1]) + d[2][2]);
 }
 
+// A field by offsets from site s; the debug build reads only inside the lattice.
+template <class R>
+struct FieldAt {
+    const R* h;  // the field at s
+    int s, n;
+    int* status;
+    __device__ __forceinline__ R operator[](int d) const { return site_ok((long long)s + d, n, status) ? h[d] : R(0); }
+};
+
 // grad mu by central differences (as unscaled differences, twice the gradient)
 // and mu at a site from phi alone: mu at the site and its six neighbours, each
 // the operations of k_mu, from the 25 phi within two sites.
 template <class R>
 __device__ __forceinline__ void mu_diffs_of_phi(const RowGeom& rg, const Model<R>& m, const R* phi, int x, int y, int z,
-                                                int s, const RowNbr& o, R& mu, R& dx, R& dy, R& dz) {
+                                                int s, const RowNbr& o, int* status, R& mu, R& dx, R& dy, R& dz) {
     const int nx = rg.nx, plane = rg.nx * rg.ny;
     const int x2 = x + 2 >= nx ? 2 - nx : 2, xm2 = x < 2 ? nx - 2 : -2;
     const int y2 = (y + 2 >= rg.ny ? 2 - rg.ny : 2) * nx, ym2 = (y < 2 ? rg.ny - 2 : -2) * nx;
     const int z2 = (z + 2 >= rg.nz ? 2 - rg.nz : 2) * plane, zm2 = (z < 2 ? rg.nz - 2 : -2) * plane;
-    const R* p = phi + s;
+    const FieldAt<R> p{phi + s, s, rg.n, status};
     const R c = p[0], xp = p[o.xp], xm = p[o.xm], yp = p[o.yp], ym = p[o.ym], zp = p[o.zp], zm = p[o.zm];
     const R xpyp = p[o.xp + o.yp], xpym = p[o.xp + o.ym], xmyp = p[o.xm + o.yp], xmym = p[o.xm + o.ym];
     const R xpzp = p[o.xp + o.zp], xpzm = p[o.xp + o.zm], xmzp = p[o.xm + o.zp], xmzm = p[o.xm + o.zm];
@@ -241,12 +250,12 @@ __device__ __forceinline__ void mu_diffs_of_phi(const RowGeom& rg, const Model<R
 // operations of k_stress, from the 25 phi within two sites.
 template <class R>
 __device__ __forceinline__ void stress_force_of_phi(const RowGeom& rg, const Model<R>& m, const R* phi, int x, int y,
-                                                    int z, int s, const RowNbr& o, R& mu, R& Fx, R& Fy, R& Fz) {
+                                                    int z, int s, const RowNbr& o, int* status, R& mu, R& Fx, R& Fy, R& Fz) {
     const int nx = rg.nx, plane = rg.nx * rg.ny;
     const int x2 = x + 2 >= nx ? 2 - nx : 2, xm2 = x < 2 ? nx - 2 : -2;
     const int y2 = (y + 2 >= rg.ny ? 2 - rg.ny : 2) * nx, ym2 = (y < 2 ? rg.ny - 2 : -2) * nx;
     const int z2 = (z + 2 >= rg.nz ? 2 - rg.nz : 2) * plane, zm2 = (z < 2 ? rg.nz - 2 : -2) * plane;
-    const R* p = phi + s;
+    const FieldAt<R> p{phi + s, s, rg.n, status};
     const R c = p[0], xp = p[o.xp], xm = p[o.xm], yp = p[o.yp], ym = p[o.ym], zp = p[o.zp], zm = p[o.zm];
     const R xpyp = p[o.xp + o.yp], xpym = p[o.xp + o.ym], xmyp = p[o.xm + o.yp], xmym = p[o.xm + o.ym];
     const R xpzp = p[o.xp + o.zp], xpzm = p[o.xp + o.zm], xmzp = p[o.xm + o.zp], xmzm = p[o.xm + o.zm];
@@ -330,11 +339,11 @@ __global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
     const R ph = phi[s];
     R muc, Fx, Fy, Fz;
     if constexpr (NEAR == kNearStress) {
-        stress_force_of_phi(rg, m, phi, x, y, z, s, o, muc, Fx, Fy, Fz);
+        stress_force_of_phi(rg, m, phi, x, y, z, s, o, status, muc, Fx, Fy, Fz);
         if (mu_out) mu_out[s] = muc;
     } else if constexpr (NEAR == kNearMu) {
         R dx, dy, dz;
-        mu_diffs_of_phi(rg, m, phi, x, y, z, s, o, muc, dx, dy, dz);
+        mu_diffs_of_phi(rg, m, phi, x, y, z, s, o, status, muc, dx, dy, dz);
         force_of_diffs(ph, dx, dy, dz, Fx, Fy, Fz);
         if (mu_out) mu_out[s] = muc;
     } else {

@@ -56,3 +56,31 @@ def test_debug_build_runs_clean_and_matches_release(ld, shape, kernel, precision
             assert np.array_equal(a, b)
         else:
             assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
+
+
+# the one-launch step of small lattices (tiles past the lattice, halos that wrap several times) and the site-ordered
+# collisions that read phi two sites away
+OPTIONS = [((4, 4, 4), "auto", "fp32", dict(stencil=7)), ((4, 4, 4), "auto", "fp32", dict(stencil=19)),
+           ((5, 9, 33), "auto", "fp32", dict(stencil=7)), ((5, 9, 33), "auto", "fp32", dict(stencil=19)),
+           ((4, 8, 32), "auto", "fp32", dict(stencil=7)), ((4, 8, 32), "auto", "fp32", dict(stencil=19)),
+           ((4, 4, 4), "auto", "fp32", dict(force="stress")), ((7, 4, 5), "auto", "fp32", dict(force="stress")),
+           ((5, 9, 33), "auto", "fp16dev", dict(force="stress", collision="trt")),
+           ((5, 4, 129), "auto", "bf16dev", dict(force="stress"))]
+
+
+@pytest.mark.parametrize("shape,kernel,precision,model", OPTIONS)
+def test_debug_build_of_small_and_near_steps(ld, shape, kernel, precision, model):
+    def run():
+        nz, ny, nx = shape
+        sim = ld.LdSim(nx, ny, nz, precision=precision, kernel=kernel, tau_f=0.9, tau_g=1.1, **model)
+        sim.init(torch.from_numpy(inputs.spinodal_phi(nx, ny, nz, seed=71, amplitude=0.3)))
+        sim.step(9)
+        sim.check()  # raises LD_ECUDA if an index left the lattice
+        return [t.cpu().numpy() for t in sim.distributions()]
+
+    release = run()
+    with ld.debug_library():
+        debug = run()
+    tol = {"fp32": 1e-6, "fp16dev": 2e-3, "bf16dev": 2e-2}[precision]
+    for a, b in zip(debug, release):
+        assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b)
