@@ -208,3 +208,56 @@ def test_fp32_crystal_initial_state_has_the_written_fusions():
     uu = fma32(u[2], u[2], fma32(u[1], u[1], u[0] * u[0]))
     for i in range(19):
         assert np.array_equal(got[i], feq32(i, rho, u, uu).astype(np.float64))
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16dev", "bf16dev"])
+@pytest.mark.parametrize("stencil", [7, 19])
+@pytest.mark.parametrize("force", ["potential", "stress"])
+def test_velocity_and_gradient_values(precision, stencil, force, orc):
+    """u = (j + F/2)/rho and grad phi in FP64 from the state's values, F from the phi, mu and P that the arithmetic
+    of the precision gives: phi and mu of the FP32 forms bit for bit, P to its rounding."""
+    nx, ny, nz = 11, 6, 5
+    rng = np.random.default_rng(21)
+    phi0, rho0 = 0.4 * rng.standard_normal((nz, ny, nx)), 1.0 + 0.05 * rng.standard_normal((nz, ny, nx))
+    u0 = 0.05 * rng.standard_normal((3, nz, ny, nx))
+    A, B, kappa = -0.07, 0.051, 0.043
+    sim = ld.LdSim(nx, ny, nz, precision=precision, stencil=stencil, force=force, A=A, B=B, kappa=kappa, tau_f=0.8)
+    sim.init(*(torch.from_numpy(a) for a in (phi0, rho0, u0)))
+    sim.step(2)
+    m = {k: v.cpu().numpy() for k, v in sim.moments(grad_phi=True).items()}
+    f, g = (t.cpu().numpy() for t in sim.distributions())  # FP32 values, or reference + deviation, exact in FP64
+    real = np.float64 if precision == "fp64" else np.float32
+    unit = 2.0 ** -53 if precision == "fp64" else 2.0 ** -24
+    phi = np.zeros((nz, ny, nx), real)
+    for i in range(19):
+        phi = phi + g[i].astype(real)
+    if stencil == 7:
+        lap = sum((np.roll(phi, s, a) for a in (2, 1, 0) for s in (-1, 1)), real(0)) - real(6) * phi
+    else:
+        lap = np.zeros_like(phi)
+        for i in range(1, 19):
+            lap = lap + real(1) / real(3 if i <= 6 else 6) * (np.roll(phi, (-C[i][2], -C[i][1], -C[i][0]), (0, 1, 2)) - phi)
+    mu = (real(A) * phi + real(B) * phi * phi * phi) - real(kappa) * lap
+    phi, mu = phi.astype(np.float64), mu.astype(np.float64)
+    exact = lambda a: np.array([math.fsum(v) for v in a.reshape(19, -1).T]).reshape(a.shape[1:])  # noqa: E731
+    c = np.array(C, float)
+    j = np.stack([exact(c[:, a, None, None, None] * f) for a in range(3)])
+    size = np.abs(f).sum(axis=0)
+    if force == "potential":
+        F = -exact(g) * orc.gradient(mu, stencil)
+        # FP32: the same mu; FP64: its own to a few units of its terms, over a gradient of weight 1
+        mu_terms = np.abs(A * phi).max() + np.abs(B * phi ** 3).max() + kappa * 12 * np.abs(phi).max()
+        f_err = 2.0 ** -53 * 64 * np.abs(phi).max() * mu_terms
+    else:
+        prm = orc.param_vector(A=float(real(A)), B=float(real(B)), kappa=float(real(kappa)), stencil=stencil, force="stress")
+        P = orc.stress(phi, prm)
+        F = -np.stack([sum(orc.gradient(P[k], stencil)[b] for b, k in enumerate(ks))
+                       for ks in ((0, 3, 4), (3, 1, 5), (4, 5, 2))])
+        # about 40 roundings of the terms of P (phi lap phi the largest), and three gradients of it
+        f_err = unit * 3 * 40 * (np.abs(P).max() + kappa * 12 * np.abs(phi).max() ** 2)
+    rho = exact(f)
+    tol = (2.0 ** -53 * 24 * (size + np.abs(F).max()) + f_err) / rho
+    assert np.abs(F).max() > 1e3 * f_err  # the force is there to be seen
+    assert (np.abs(m["u"] - (j + 0.5 * F) / rho) <= tol).all()
+    phi_err = 0.0 if precision != "fp64" else 18 * 2.0 ** -53 * np.abs(g).sum(axis=0).max()
+    assert np.abs(m["grad_phi"] - orc.gradient(phi, stencil)).max() <= 16 * 2.0 ** -53 * np.abs(phi).max() + phi_err
