@@ -423,8 +423,8 @@ __device__ __forceinline__ double div_by(double n, double d, double inv) {
     return __fma_rn(__fma_rn(-q, d, n), inv, q);
 }
 __device__ __forceinline__ bool any_nonfinite(double a, double b, double c) {
-    const int ea = __double2hiint(a) & 0x7fffffff, eb = __double2hiint(b) & 0x7fffffff, ec = __double2hiint(c) & 0x7fffffff;
-    return max(max(ea, eb), ec) >= 0x7ff00000;
+    const int ma = __double2hiint(a) & 0x7fffffff, mb = __double2hiint(b) & 0x7fffffff;
+    return max(max(ma, mb), __double2hiint(c) & 0x7fffffff) >= 0x7ff00000;
 }
 __device__ __forceinline__ void guo_velocity(double rho, double jx, double jy, double jz, double Fx, double Fy,
                                              double Fz, double& ux, double& uy, double& uz) {

@@ -240,7 +240,8 @@ def ld_unpack_planes(ctx, z0: int, nplanes: int, buf):
 
 
 def ld_step_kernel(ctx) -> str:
-    """Name of the step kernel the context runs (AUTO resolved)."""
+    """Name of the step kernel the context runs (AUTO resolved; where AUTO runs its small-lattice kernel, the one it
+    resolves to on larger lattices of the same divisibility, with the same results)."""
     code = lib().ld_step_kernel(ctx)
     names = {v: k for k, v in KERNELS.items()}
     if code not in names:
