@@ -284,32 +284,43 @@ __device__ __forceinline__ void stress_force_of_phi(const RowGeom& rg, const Mod
 }
 
 // How the step's collision comes by mu and the force: from the fields that
-// k_mu or k_stress wrote (kFar), or from phi itself, without those launches:
-// kNearMu with the potential force, kNearStress with the stress force. The
-// near forms take the 7-point stencils (the 19-point ones would need 19 phi
-// at each of 18 neighbours) and FP32 arithmetic (in FP64 they would add 60 and
-// 200 instructions to the pipe that bounds the step).
-enum { kFar = 0, kNearMu = 1, kNearStress = 2 };
+// k_mu or k_stress wrote (kFar; kFarStress in FP32 storage with the stress
+// force), or from phi itself, without those launches: kNearMu with the
+// potential force, kNearStress with the stress force. The near forms take the
+// 7-point stencils (the 19-point ones would need 19 phi at each of 18
+// neighbours) and FP32 arithmetic (in FP64 they would add 60 and 200
+// instructions to the pipe that bounds the step), so FP32 comes to the far
+// ones with the 19-point stencils only. One FP32 kernel for both forces and
+// either stencil held its 38 early loads through all of it and spilled: the
+// stress force at 192^3 took 762 us a step (four launches a step before: 708),
+// in a kernel of its own 640. The 16-bit forms load g after the f stores.
+enum { kFar = 0, kNearMu = 1, kNearStress = 2, kFarStress = 3 };
+__host__ __device__ constexpr bool is_near(int form) { return form == kNearMu || form == kNearStress; }
 template <int P>
-int near_form(const ld_ctx* c) {
-    if (sizeof(typename Prec<P>::real_t) == 8 || c->prm.stencil != LD_STENCIL_7) return kFar;
-    return c->stress ? kNearStress : kNearMu;
+__host__ __device__ constexpr bool far_stress_apart() {
+    return sizeof(typename Prec<P>::store_t) == 4;
+}
+template <int P>
+int collide_form(const ld_ctx* c) {
+    if (sizeof(typename Prec<P>::real_t) == 8) return kFar;
+    if (c->prm.stencil == LD_STENCIL_7) return c->stress ? kNearStress : kNearMu;
+    return far_stress_apart<P>() && c->stress ? kFarStress : kFar;
 }
 
-// Resident blocks per SM the collision kernel is compiled for: 6 x 128
-// threads (80 registers) with FP32 arithmetic, 5 (96) where it forms mu from
-// phi, 3 with FP64.
-template <int P, int NEAR>
+// Resident blocks per SM the collision kernel is compiled for: with FP32
+// arithmetic 6 x 128 threads (80 registers), 5 (96) where it forms mu from phi;
+// 3 with FP64.
+template <int P, int FORM>
 constexpr int rows_blocks_per_sm() {
-    return sizeof(typename Prec<P>::real_t) == 4 ? (NEAR != kFar ? 5 : 6) : 3;
+    return sizeof(typename Prec<P>::real_t) == 4 ? (is_near(FORM) ? 5 : 6) : 3;
 }
 
 // Stage 3: force, velocity, collisions of f and g, and propagation (push: the
 // post-collision value of direction i goes to x + c_i) with streaming stores;
-// NEAR: where mu and the force come from (near forms write mu to mu_out when
+// FORM: where mu and the force come from (near forms write mu to mu_out when
 // it is not null); SR: the 16-bit stores rounded stochastically from `sr`.
-template <int P, class I, int NEAR, bool SR>
-__global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
+template <int P, class I, int FORM, bool SR>
+__global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, FORM>()))
     k_collide(RowGeom rg, I npad, Model<typename Prec<P>::real_t> m, SrStream sr, const typename Prec<P>::store_t* __restrict__ fs,
               const typename Prec<P>::store_t* __restrict__ gs, typename Prec<P>::store_t* __restrict__ fd,
               typename Prec<P>::store_t* __restrict__ gd, const typename Prec<P>::real_t* __restrict__ phi,
@@ -338,19 +349,21 @@ __global__ void __launch_bounds__(kRowThreads, (rows_blocks_per_sm<P, NEAR>()))
     const int oxp = o.xp, oxm = o.xm, oyp = o.yp, oym = o.ym, ozp = o.zp, ozm = o.zm;
     const R ph = phi[s];
     R muc, Fx, Fy, Fz;
-    if constexpr (NEAR == kNearStress) {
+    if constexpr (FORM == kNearStress) {
         stress_force_of_phi(rg, m, phi, x, y, z, s, o, status, muc, Fx, Fy, Fz);
         if (mu_out) mu_out[s] = muc;
-    } else if constexpr (NEAR == kNearMu) {
+    } else if constexpr (FORM == kNearMu) {
         R dx, dy, dz;
         mu_diffs_of_phi(rg, m, phi, x, y, z, s, o, status, muc, dx, dy, dz);
         force_of_diffs(ph, dx, dy, dz, Fx, Fy, Fz);
         if (mu_out) mu_out[s] = muc;
     } else {
+        constexpr bool kApart = far_stress_apart<P>();
+        const int iso = kApart ? 1 : m.iso;
         muc = mu[s];
-        if (stress) {  // F = -div P
-            stress_force_at(m.iso, stress, npad, s, o, Fx, Fy, Fz);
-        } else if (m.iso) {  // F = -phi grad(mu)
+        if (kApart ? FORM == kFarStress : stress != nullptr) {  // F = -div P
+            stress_force_at(iso, stress, npad, s, o, Fx, Fy, Fz);
+        } else if (iso) {  // F = -phi grad(mu)
             R gmx, gmy, gmz;
             grad_at(1, mu, s, o, gmx, gmy, gmz);
             Fx = -ph * gmx, Fy = -ph * gmy, Fz = -ph * gmz;
@@ -898,33 +911,35 @@ cudaError_t phi_mu_p(ld_ctx* c, const void* state) {
 
 // One step; phi and mu of the source state go to `fields` ([phi npad][mu
 // npad]) when it is not null, else to the context's scratch.
-template <int P, class I, int NEAR, bool SR>
+template <int P, class I, int FORM, bool SR>
 cudaError_t collide_rows(ld_ctx* c, const void* src, void* dst, void* fields) {
     using S = typename Prec<P>::store_t;
     using R = typename Prec<P>::real_t;
     R* phi = fields ? (R*)fields : (R*)c->phi;
     R* mu = fields ? (R*)fields + c->geom.npad : (R*)c->mu;
     launch_phi<P, I>(c, src, phi);
-    if (NEAR == kFar) launch_mu<R, I>(c, phi, mu);
-    k_collide<P, I, NEAR, SR><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
+    if (!is_near(FORM)) launch_mu<R, I>(c, phi, mu);
+    k_collide<P, I, FORM, SR><<<row_blocks(c->geom), kRowThreads, 0, c->stream>>>(
         row_geom(c->geom), (I)c->geom.npad, model_of<R>(c->prm), sr_stream(c->prm.seed, c->sr_step, c->geom.n),
         (const S*)f_part(c, src), (const S*)g_part(c, src), (S*)f_part(c, dst), (S*)g_part(c, dst), phi,
-        NEAR != kFar ? nullptr : mu, c->ref, (const R*)c->stress, NEAR != kFar && fields ? mu : nullptr, c->status);
+        is_near(FORM) ? nullptr : mu, c->ref, (const R*)c->stress, is_near(FORM) && fields ? mu : nullptr, c->status);
     return cudaGetLastError();
 }
 
-template <int P, int NEAR, bool SR>
+template <int P, int FORM, bool SR>
 cudaError_t collide_r(ld_ctx* c, const void* src, void* dst, void* fields) {
-    return offsets_fit_int(c) ? collide_rows<P, int, NEAR, SR>(c, src, dst, fields)
-                              : collide_rows<P, long long, NEAR, SR>(c, src, dst, fields);
+    return offsets_fit_int(c) ? collide_rows<P, int, FORM, SR>(c, src, dst, fields)
+                              : collide_rows<P, long long, FORM, SR>(c, src, dst, fields);
 }
 
 template <int P, bool SR>
 cudaError_t collide_n(ld_ctx* c, const void* src, void* dst, void* fields) {
     if constexpr (sizeof(typename Prec<P>::real_t) == 4) {
-        switch (near_form<P>(c)) {
+        switch (collide_form<P>(c)) {
             case kNearMu: return collide_r<P, kNearMu, SR>(c, src, dst, fields);
             case kNearStress: return collide_r<P, kNearStress, SR>(c, src, dst, fields);
+            case kFarStress:
+                if constexpr (far_stress_apart<P>()) return collide_r<P, kFarStress, SR>(c, src, dst, fields);
         }
     }
     return collide_r<P, kFar, SR>(c, src, dst, fields);

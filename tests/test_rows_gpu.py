@@ -77,12 +77,13 @@ def test_adjoint_step_from_an_unaligned_state(precision):
 @pytest.mark.parametrize("dims", [(4, 4, 4), (5, 4, 7), (33, 9, 5), (129, 6, 4)])
 @pytest.mark.parametrize("precision", ["fp32", "fp16dev", "bf16dev"])
 @pytest.mark.parametrize("collision", ["bgk", "trt"])
-def test_stress_force_formed_in_the_collision(dims, precision, collision, orc):
+@pytest.mark.parametrize("stencil", [7, 19])
+def test_one_step_with_the_stress_force(dims, precision, collision, stencil, orc):
     """One step with F = -div P from a stored state in flow, against the oracle's from the same state, and the
-    fields it leaves. Dimensions of 4 and 5, where +2 and -2 meet or wrap, and blocks across the ends of rows."""
+    fields it leaves: formed in the collision (7-point) and from the stress launch (19-point). Dimensions of 4 and 5, where +2 and -2 meet or wrap, and blocks across the ends of rows."""
     nx, ny, nz = dims
     n, npad = nx * ny * nz, -(-nx * ny * nz // 64) * 64
-    sim = started(nx, ny, nz, precision=precision, force="stress", collision=collision)
+    sim = started(nx, ny, nz, precision=precision, force="stress", collision=collision, stencil=stencil)
     phi0 = inputs.spinodal_phi(nx, ny, nz, seed=8, amplitude=0.5)
     sim.step(2)
     f0, g0 = (t.cpu().numpy() for t in sim.distributions())
@@ -95,18 +96,25 @@ def test_stress_force_formed_in_the_collision(dims, precision, collision, orc):
     phi, mu = (a[:n].view(nz, ny, nx).cpu().numpy() for a in fld.view(torch.float32)[:2 * npad].view(2, npad))
     # phi: 18 roundings of the magnitudes (19 more where the values are decoded); mu: the operations of the mu launch
     assert (np.abs(phi - g0.sum(axis=0)) <= 38 * 2.0 ** -24 * np.abs(g0).sum(axis=0)).all()
-    nb = np.zeros_like(phi)
-    for axis in (2, 1, 0):
-        nb = nb + np.roll(phi, -1, axis) if axis < 2 else np.roll(phi, -1, axis)
-        nb = nb + np.roll(phi, 1, axis)
+    c, w = orc.lattice()
+    one = np.float32(1)
+    if stencil == 7:
+        nb = np.zeros_like(phi)
+        for axis in (2, 1, 0):
+            nb = nb + np.roll(phi, -1, axis) if axis < 2 else np.roll(phi, -1, axis)
+            nb = nb + np.roll(phi, 1, axis)
+        lap = nb - np.float32(6) * phi
+    else:
+        lap = np.zeros_like(phi)
+        for i in range(1, 19):
+            lap = lap + one / np.float32(3 if i <= 6 else 6) * (np.roll(phi, -c[i][::-1], (0, 1, 2)) - phi)
     A, B, kappa = (np.float32(v) for v in (-0.0625, 0.0625, 0.05))
-    assert np.array_equal(mu, (A * phi + B * phi * phi * phi) - kappa * (nb - np.float32(6) * phi))
-    prm = orc.param_vector(**dict(MODEL, kappa=float(kappa)), force="stress", collision=collision)
+    assert np.array_equal(mu, (A * phi + B * phi * phi * phi) - kappa * lap)
+    prm = orc.param_vector(**dict(MODEL, kappa=float(kappa)), force="stress", collision=collision, stencil=stencil)
     want = np.concatenate(orc.step(f0, g0, prm))
     # FP32: about 60 operations reach a population, on terms no larger than the density
     tol = 64 * 2.0 ** -24 * f0.sum(axis=0).max()
     if precision != "fp32":  # and half a unit of the stored deviation
-        c, w = orc.lattice()
         pb = phi0.mean()
         dev = 0.5 * (-0.0625 * pb + 0.0625 * pb ** 3) - pb / 3
         ref = np.concatenate([w, w * (pb + 4.5 * dev * ((c ** 2).sum(axis=1) - 1))])[:, None, None, None]
