@@ -34,6 +34,16 @@ namespace ld {
 namespace {
 
 constexpr int kAdjThreads = 256;
+// Blocks of one site per thread that are resident at once, 8 on each of 152 SMs:
+// up to here k_adj_mu takes one site a thread and the final pass 256 threads,
+// since the latency of one thread's serial sites is the launch's time; beyond
+// it four sites and 1024 threads. Measured, us of k_adj_mu with four and with
+// one (19-point in brackets): 16^3 5.0 and 2.5 (6.7 and 3.8), 32^3 5.5 and 2.7
+// (7.8 and 4.2), 64^3 7.1 and 6.5 (10.0 and 8.3), 80^3 9.0 and 10.6 (12.8 and
+// 14.4), 128^3 27 and 33 (44 and 47), FP64 19-point at 32^3 33 and 10; of the
+// final pass with 1024 and with 256 threads: 32^3 3.4 and 2.2, 64^3 3.7 and 3.1,
+// 80^3 4.8 and 5.2, 128^3 7.0 and 8.6.
+constexpr int kAdjOneWave = 8 * 152;
 
 // Fixed-order block sum of one double per thread into out[0]: the first warp
 // adds the others' values, eight per lane, then its lanes. The FP64 pipe takes
@@ -196,20 +206,18 @@ struct ProductSum<float> {
     __device__ __forceinline__ double value() const { return rest + ((double)a.s + ((double)a.e + (double)a.t)); }
 };
 
-// Sites per thread of k_adj_mu, kAdjThreads apart.
-constexpr int kAdjMuSites = 4;
-
 // Step 3: mubar += transpose of the gradient applied to gmbar; kappa
 // partials mubar (-lap phi). 7-point: the transposed central difference;
-// 19-point: mubar(y) += sum_i 3 w_i c_i . gmbar(y - c_i).
-template <class R, class I, bool ISO>
+// 19-point: mubar(y) += sum_i 3 w_i c_i . gmbar(y - c_i). SITES sites per
+// thread, kAdjThreads apart.
+template <class R, class I, bool ISO, int SITES>
 __global__ void __launch_bounds__(kAdjThreads)
     k_adj_mu(RowGeom rg, I npad, const R* __restrict__ phi, const R* __restrict__ gmb, R* __restrict__ mub,
              double* __restrict__ part) {
     ProductSum<R> kappa_bar;
 #pragma unroll
-    for (int k = 0; k < kAdjMuSites; ++k) {
-        const int s = (int)((blockIdx.x * kAdjMuSites + k) * kAdjThreads + threadIdx.x);
+    for (int k = 0; k < SITES; ++k) {
+        const int s = (int)((blockIdx.x * SITES + k) * kAdjThreads + threadIdx.x);
         if ((unsigned)s >= (unsigned)rg.n) break;
         const RowNbr o = site_nbr(rg, s);
         const R *gx = gmb + s, *gy = gmb + npad + s, *gz = gmb + 2 * npad + s;
@@ -263,17 +271,17 @@ __global__ void __launch_bounds__(kAdjThreads)
 // grad[0] += the sum of part[2b + 1] over b < nkappa (kappa); grad[1] +=
 // taub_scale * the sum of part[2b] over b < ntau (tau_f); one block, fixed
 // order.
-constexpr int kAdjFinalThreads = 1024;
-__global__ void __launch_bounds__(kAdjFinalThreads)
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS)
     k_adj_finalize(const double* __restrict__ part, int nkappa, int ntau, double taub_scale, double* __restrict__ grad) {
     // One block's sums run on one SM's FP64 pipe: a warp for each of the two
     // adds the other warps' values (a shuffle tree in all 32 warps and a serial
     // pass over them took 11 us).
-    __shared__ double red[2][kAdjFinalThreads];
+    __shared__ double red[2][THREADS];
     double a = 0.0, b = 0.0;
-    for (int k = threadIdx.x; k < nkappa; k += kAdjFinalThreads) a += part[2 * (long long)k + 1];
+    for (int k = threadIdx.x; k < nkappa; k += THREADS) a += part[2 * (long long)k + 1];
 #pragma unroll 8
-    for (int k = threadIdx.x; k < ntau; k += kAdjFinalThreads) b += part[2 * (long long)k];
+    for (int k = threadIdx.x; k < ntau; k += THREADS) b += part[2 * (long long)k];
     red[0][threadIdx.x] = a;
     red[1][threadIdx.x] = b;
     __syncthreads();
@@ -281,10 +289,16 @@ __global__ void __launch_bounds__(kAdjFinalThreads)
     if (warp > 1) return;
     double v[4] = {0.0, 0.0, 0.0, 0.0};  // four chains: the additions' latency, not their number, is what waits
 #pragma unroll
-    for (int w = 0; w < kAdjFinalThreads / 32; ++w) v[w & 3] += red[warp][lane + 32 * w];
+    for (int w = 0; w < THREADS / 32; ++w) v[w & 3] += red[warp][lane + 32 * w];
     double t = (v[0] + v[1]) + (v[2] + v[3]);
     for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
     if (lane == 0) grad[warp] += warp == 0 ? t : taub_scale * t;
+}
+inline void launch_adj_finalize(const ld_ctx* c, int nkappa, int ntau, double taub_scale, double* grad) {
+    if (ntau <= kAdjOneWave)
+        k_adj_finalize<256><<<1, 256, 0, c->stream>>>(c->adj_part, nkappa, ntau, taub_scale, grad);
+    else
+        k_adj_finalize<1024><<<1, 1024, 0, c->stream>>>(c->adj_part, nkappa, ntau, taub_scale, grad);
 }
 
 // Seed: fbar = 0, gbar_i = phibar (the adjoint of phi_T = sum_i g_i), i.e.
@@ -412,15 +426,16 @@ cudaError_t adj_step_iso(ld_ctx* c, const void* state_t, const void* fields_t, d
     const R* mu = fields_t ? (const R*)fields_t + c->geom.npad : (const R*)c->mu;
     const AdjPtrs<P> p = adj_ptrs<P>(c, c->adj_cur);
     const Model<R> m = model_of<R>(c->prm);
-    const unsigned nb = blocks_for(c->geom.n), nbm = (nb + kAdjMuSites - 1) / kAdjMuSites;
+    const unsigned nb = blocks_for(c->geom.n), per = nb <= kAdjOneWave ? 1 : 4, nbm = (nb + per - 1) / per;
     k_adj_local<P, I, ISO><<<nb, kAdjThreads, 0, c->stream>>>(rg, npad, m, (const S*)f_part(c, state_t), phi, mu, c->ref,
                                                               p.fb1, p.gb1, p.pb1, p.fb0, p.gb0, p.gmb, p.mub, p.phib,
                                                               c->adj_part);
-    k_adj_mu<R, I, ISO><<<nbm, kAdjThreads, 0, c->stream>>>(rg, npad, phi, p.gmb, p.mub, c->adj_part);
+    if (per == 1)
+        k_adj_mu<R, I, ISO, 1><<<nbm, kAdjThreads, 0, c->stream>>>(rg, npad, phi, p.gmb, p.mub, c->adj_part);
+    else
+        k_adj_mu<R, I, ISO, 4><<<nbm, kAdjThreads, 0, c->stream>>>(rg, npad, phi, p.gmb, p.mub, c->adj_part);
     k_adj_p<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(rg, m, phi, p.mub, p.phib, p.pb0);
-    if (grad)
-        k_adj_finalize<<<1, kAdjFinalThreads, 0, c->stream>>>(c->adj_part, (int)nbm, (int)nb,
-                                                              -1.0 / (c->prm.tau_f * c->prm.tau_f), grad);
+    if (grad) launch_adj_finalize(c, (int)nbm, (int)nb, -1.0 / (c->prm.tau_f * c->prm.tau_f), grad);
     return cudaGetLastError();
 }
 
@@ -454,7 +469,7 @@ cudaError_t adj_init_iso(ld_ctx* c, const double* phi0, const double* u0, double
     k_adj_init_mu<R><<<nb, kAdjThreads, 0, c->stream>>>(g, (R)c->prm.Gamma, p.gb1, p.pb1, p.mub);
     k_adj_init_phi<R, ISO><<<nb, kAdjThreads, 0, c->stream>>>(g, row_geom(c->geom), model_of<R>(c->prm), phi0, u0, p.gb1, p.pb1, p.mub,
                                                          grad_phi0, c->adj_part);
-    if (grad) k_adj_finalize<<<1, kAdjFinalThreads, 0, c->stream>>>(c->adj_part, (int)nb, (int)nb, 0.0, grad);
+    if (grad) launch_adj_finalize(c, (int)nb, (int)nb, 0.0, grad);
     return cudaGetLastError();
 }
 
