@@ -442,9 +442,17 @@ __global__ void __launch_bounds__(kLcThreads) k_lc_collide(LcGeom g, LcModel<T> 
 }
 
 // RECOMPUTE_H: form H from Q here (the fused step stores no H) instead of
-// reading the h written by k_lc_field; the same arithmetic either way.
+// reading the h written by k_lc_field; the same arithmetic either way. In FP32
+// the launch waits on its loads and is compiled for 9 blocks per SM (56
+// registers; left alone, 70 with H recomputed): us at 256^3 as the second
+// launch of the fused step 314 before and 289 so, after the per-site launches
+// 339 and 310 (8 blocks 295 and 316; 10 blocks spill with H, 354 and 329).
+template <class T>
+__host__ __device__ constexpr int lc_update_blocks() {
+    return sizeof(T) == 4 ? 9 : 0;  // 0: no minimum
+}
 template <class T, bool RECOMPUTE_H>
-__global__ void __launch_bounds__(kLcThreads) k_lc_update(LcGeom g, LcModel<T> m, const T* __restrict__ q,
+__global__ void __launch_bounds__(kLcThreads, lc_update_blocks<T>()) k_lc_update(LcGeom g, LcModel<T> m, const T* __restrict__ q,
                                                           const T* __restrict__ u, const T* __restrict__ h,
                                                           T* __restrict__ qn) {
     LcSite t;
